@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(1024) k_batch_sweep(const BatchArgs b)
     __shared__ uint4 s_tab[dev::kThresholdEntries];
     __shared__ int s_prefix[kMaxRuns + 1];
     __shared__ int s_group;
-    __shared__ uint32_t s_queue[dev::queue_words(PART == 0 ? 4 : 7)];
+    __shared__ __align__(16) uint32_t s_queue[dev::queue_words(PART == 0 ? 4 : 7)];
     const int i = *b.step_counter;
     int *work = b.work + PART * b.work_stride + i;
     if (threadIdx.x == 0) {

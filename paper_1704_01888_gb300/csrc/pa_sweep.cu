@@ -73,13 +73,13 @@ __device__ __forceinline__ dev::Group make_group(const SweepArgs &a, int parity,
 // B: bits per state; MODE: 0 for L = 64, 1 for L a multiple of 64, 3 for
 // L = 8, 16, 32 (rows packed several to a word), 4 for L = 48, 80, 96, ...
 // (banded 8-column segments), 2 otherwise (rows padded to whole words).
-template <int B, int MODE, int Q>
-__global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a)
+template <int B, int MODE, int Q, bool LAT>
+__device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
 {
     extern __shared__ uint4 smem4[];
     __shared__ uint4 s_tab[dev::kThresholdEntries];
-    constexpr int QCAP = B <= 4 ? 384 : dev::kQueueCap;
-    __shared__ uint32_t s_queue[dev::queue_words(B, QCAP)];
+    constexpr int QCAP = LAT ? dev::kLatQueue : B <= 4 ? 384 : dev::kQueueCap;
+    __shared__ __align__(16) uint32_t s_queue[dev::queue_words(B, QCAP)];
     dev::build_threshold_table(s_tab, a.thr);
     DevState *st = a.st;
     if (st->err) return;
@@ -102,10 +102,16 @@ __global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a)
         }
         if (first >= end) break;
         const dev::Group G = make_group(a, parity, first, min(a.rpb, end - first));
-        dev::sweep_group_bits<B, MODE, Q, MODE == 0 || MODE == 1, QCAP, MODE != 0>(
+        dev::sweep_group_bits<B, MODE, Q, QCAP, LAT>(
             G, a.L, reinterpret_cast<uint32_t *>(smem4), s_tab, s_queue, a.rk0, a.rk1, sE, sE2, sM);
     }
     if ((threadIdx.x & 31) == 0 && (sE | sE2 | sM)) dev::accumulate_totals(a.acc, sE, sE2, sM);
+}
+
+template <int B, int MODE, int Q>
+__global__ void __launch_bounds__(1024) k_sweep(const SweepArgs a)
+{
+    sweep_blocks<B, MODE, Q, false>(a);
 }
 
 // Allows each kernel the device's full opt-in shared memory (less its static

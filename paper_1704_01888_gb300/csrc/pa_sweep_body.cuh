@@ -122,7 +122,8 @@ __device__ __forceinline__ uint32_t shifted_row(uint32_t H, uint32_t E, int par,
     } else if constexpr (MODE == 1) {
         return par ? __funnelshift_r(H, E, 1) : __funnelshift_r(E, H, 31);
     } else {
-        return par ? ((H >> 1) | ((E & 1u) << (nb - 1))) : ((H << 1) | ((E >> (nbe - 1)) & 1u));
+        // bits past a row's columns are zero in E and not looked at in the result
+        return par ? ((H >> 1) | (E << (nb - 1))) : ((H << 1) | (E >> (nbe - 1)));
     }
 }
 
@@ -131,20 +132,32 @@ __device__ __forceinline__ uint32_t shifted_row(uint32_t H, uint32_t E, int par,
 // odd x (par = 1) the neighbour not at the same column is column m + 1, else
 // m - 1, both cyclic within the row's S-bit segment.  Rows alternate par, and
 // `odd` marks the segments with par = 1 (the same in every word of a colour).
-template <int S>
-__device__ __forceinline__ uint32_t shifted_packed(uint32_t H, uint32_t odd)
+// L = 8 (four-bit rows): masked shifts.
+__device__ __forceinline__ uint32_t shifted_nibbles(uint32_t H, uint32_t odd)
 {
-    constexpr uint32_t bot = S == 4 ? 0x11111111u : S == 8 ? 0x01010101u : 0x00010001u;
-    constexpr uint32_t top = bot << (S - 1);
-    const uint32_t right = ((H >> 1) & ~top) | ((H << (S - 1)) & top);  // column m + 1
-    const uint32_t left = ((H << 1) & ~bot) | ((H >> (S - 1)) & bot);   // column m - 1
+    constexpr uint32_t bot = 0x11111111u, top = bot << 3;
+    const uint32_t right = ((H >> 1) & ~top) | ((H << 3) & top);  // column m + 1
+    const uint32_t left = ((H << 1) & ~bot) | ((H >> 3) & bot);   // column m - 1
     return (odd & right) | (~odd & left);
 }
 
-template <int S>
-__device__ __forceinline__ constexpr uint32_t odd_segments()
+// L = 16 and 32 (rows of one or two bytes): the rows that take column m - 1
+// are doubled side by side (byte selector l) and shifted left, the others (r)
+// doubled and shifted right, so that each row's wrapped bit arrives from its
+// copy; `out` picks the rows' bytes: five instructions per plane against
+// eight with masks.
+struct RowSelectors {
+    uint32_t l, r, out;
+};
+__device__ __forceinline__ RowSelectors row_selectors(int L, int c)
 {
-    return S == 4 ? 0xF0F0F0F0u : S == 8 ? 0xFF00FF00u : 0xFFFF0000u;
+    if (L == 32) return c ? RowSelectors{0x3232u, 0x1010u, 0x3254u} : RowSelectors{0x1010u, 0x3232u, 0x5432u};
+    return c ? RowSelectors{0x3311u, 0x2200u, 0x3614u} : RowSelectors{0x2200u, 0x3311u, 0x6341u};
+}
+__device__ __forceinline__ uint32_t shifted_bytes(uint32_t H, const RowSelectors &sel)
+{
+    const uint32_t l = __byte_perm(H, 0u, sel.l) << 1, r = __byte_perm(H, 0u, sel.r) >> 1;
+    return __byte_perm(l, r, sel.out);
 }
 
 // The four neighbour words of site word `it` (its index within its colour) of
@@ -193,19 +206,21 @@ __device__ __forceinline__ uint32_t neighbour_planes(const uint32_t *oth, int L,
         load_planes<BP>(H, oth + it * BP);
         load_planes<BP>(Hu, oth + wu * BP);
         load_planes<BP>(Hd, oth + wd * BP);
-        auto body = [&](auto S_tag) {
-            constexpr int S = decltype(S_tag)::value;
-            const uint32_t seg = c ? ~odd_segments<S>() : odd_segments<S>();
+        const int S = L >> 1;
 #pragma unroll
-            for (int p = 0; p < B; ++p) {
-                U[p] = (H[p] << S) | (Hu[p] >> (32 - S));
-                D[p] = (H[p] >> S) | (Hd[p] << (32 - S));
-                X[p] = shifted_packed<S>(H[p], seg);
-            }
-        };
-        if (L == 8) body(std::integral_constant<int, 4>{});
-        else if (L == 16) body(std::integral_constant<int, 8>{});
-        else body(std::integral_constant<int, 16>{});
+        for (int p = 0; p < B; ++p) {
+            U[p] = __funnelshift_l(Hu[p], H[p], S);
+            D[p] = __funnelshift_r(H[p], Hd[p], S);
+        }
+        if (L == 8) {
+            const uint32_t seg = c ? 0x0F0F0F0Fu : 0xF0F0F0F0u;
+#pragma unroll
+            for (int p = 0; p < B; ++p) X[p] = shifted_nibbles(H[p], seg);
+        } else {
+            const RowSelectors sel = row_selectors(L, c);
+#pragma unroll
+            for (int p = 0; p < B; ++p) X[p] = shifted_bytes(H[p], sel);
+        }
         return 0xFFFFFFFFu;
     } else {
         const int y = MODE == 0 ? it : div_by(it, inv_row);
@@ -231,25 +246,6 @@ __device__ __forceinline__ uint32_t neighbour_planes(const uint32_t *oth, int L,
             return valid_mask(t, WPR, nb_last);
         }
     }
-}
-
-// Block-wide sum of ints; every thread receives it.  All threads must call.
-__device__ __forceinline__ int block_sum_int(int v)
-{
-    __shared__ int s_red[33];
-    v = __reduce_add_sync(0xFFFFFFFFu, v);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) s_red[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        int x = lane < (int)(blockDim.x >> 5) ? s_red[lane] : 0;
-        x = __reduce_add_sync(0xFFFFFFFFu, x);
-        if (lane == 0) s_red[32] = x;
-    }
-    __syncthreads();
-    const int r = s_red[32];
-    __syncthreads();
-    return r;
 }
 
 // ===========================================================================
@@ -311,22 +307,28 @@ __device__ __forceinline__ void group_families(const Group &G)
 constexpr int kThresholdEntries = 41;
 constexpr int kThresholdFull = 40;
 
-// Two-pass acceptance.  In the first pass every site word draws at most
-// kFirstPassCalls Philox calls of acceptance words (the warp stops early when
-// all its sites are decided); a word with sites still undecided after that
-// (about 8 % of words at low temperature) goes to a block-wide queue, and in
-// the second pass whole warps serve only queued words, so a warp no longer
-// waits for the slowest of its ~700 sites.  Queue layout in shared memory:
-// two counters, QCAP entries of (site-word index, outcome bits acc,
-// undecided, class bits c0, e1, B proposal planes).  A full queue is not an error: the
-// word's own thread finishes it.  The single-run kernel with up to four planes
-// takes 384 entries (its 48 lattices give up to ~250 queued words at low
-// temperature, so 256 entries overflowed: 1846 against 1837 attempts/ns over
-// the at-scale schedule; two blocks per SM still fit); the batched kernel
+// Two-pass acceptance.  In the first pass every site word draws exactly
+// kFirstPassCalls Philox calls of acceptance words; a word with sites still
+// undecided after that (about 8 % of words at low temperature) goes to a
+// block-wide queue, and in the second pass whole warps serve only queued
+// words, so a warp does not wait for the slowest of its ~700 sites.  (No vote
+// before the first-pass calls: a call is skipped only if all 1024 sites of a
+// warp are decided, which half of the open sites per plane all but rules
+// out.)  The word itself is written with its decided sites in the first
+// pass; the queue entry keeps what the second pass needs for the others:
+// {word index, undecided, class bits c0, e1, B proposal planes}, padded to
+// whole 16-byte vectors, after two counters.  A full queue is not an error:
+// the word's own thread finishes it.  The single-run kernel with up to four
+// planes takes 384 entries (its 48 lattices give up to ~250 queued words at
+// low temperature, so 256 entries overflowed: 1846 against 1837 attempts/ns
+// over the at-scale schedule; two blocks per SM still fit); the batched kernel
 // keeps 256, whose 96 KB lattice budget two blocks per SM would not fit with more.
 constexpr int kFirstPassCalls = 2;
+constexpr int kLatCalls = 3;
+constexpr int kLatQueue = 90;
 constexpr int kQueueCap = 256;
-__host__ __device__ constexpr int queue_words(int B, int cap = kQueueCap) { return 2 + (5 + B) * cap; }
+__host__ __device__ constexpr int queue_entry_words(int B) { return (4 + B + 3) & ~3; }
+__host__ __device__ constexpr int queue_words(int B, int cap = kQueueCap) { return 4 + queue_entry_words(B) * cap; }
 // Entry j holds, for the threshold bits t_1..t_4 of plane j (bit 31 - j of
 // T[1..4]), the coefficients of two multiply-adds: c0 * (t_1 - t_2) - t_2
 // gives the threshold bits of the dE = 1, 2 sites (c0: dE odd) and
@@ -371,49 +373,158 @@ __device__ __forceinline__ void acceptance_plane(uint32_t v_bits, int j, const u
     und &= ~(v_bits ^ tj);
 }
 
+// ---- Philox calls of the sweep, the first rounds shared ------------------
+// The sweep's counters (w, ctr, step, slot) differ between the calls of a word
+// only in ctr (sweep, colour, call number), between the replicas only in
+// slot.  Followed through the rounds: round 0's products depend on w and on
+// step, round 1's on ctr and on (w, slot), round 2's on (w, slot) and on
+// (w, ctr).  So of a call's twenty products only the fourteen of rounds 3..9
+// belong to the call alone; two are made once per word (PhiloxWord) and one
+// once per word index and counter (PhiloxCtr), which a thread that keeps one
+// word index through its replicas makes once per half sweep.
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
+
+struct PhiloxWord {
+    uint32_t y, z, w;  // state words after round 2, less the parts that follow ctr (z: without w2)
+};
+struct PhiloxCtr {
+    uint32_t x, y, w2;  // x: without PhiloxWord::y
+};
+
+__device__ __forceinline__ PhiloxWord philox_word(uint32_t w, uint32_t step, uint32_t slot, const uint32_t *rk0,
+                                                  const uint32_t *rk1)
+{
+    const uint32_t z1 = __umulhi(kPhiloxM0, w) ^ slot ^ rk1[0];
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * z1;
+    const uint32_t x2 = (uint32_t)(p1 >> 32) ^ (kPhiloxM1 * step) ^ rk0[1];
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * x2;
+    return {(uint32_t)p1, (uint32_t)(p0 >> 32) ^ rk1[2], (uint32_t)p0};
+}
+
+__device__ __forceinline__ PhiloxCtr philox_ctr(uint32_t w, uint32_t ctr, uint32_t step, const uint32_t *rk0,
+                                                const uint32_t *rk1)
+{
+    const uint32_t x1 = __umulhi(kPhiloxM1, step) ^ ctr ^ rk0[0];
+    const uint64_t p0 = (uint64_t)kPhiloxM0 * x1;
+    const uint32_t z2 = (uint32_t)(p0 >> 32) ^ (kPhiloxM0 * w) ^ rk1[1];
+    const uint64_t p1 = (uint64_t)kPhiloxM1 * z2;
+    return {(uint32_t)(p1 >> 32) ^ rk0[2], (uint32_t)p1, (uint32_t)p0};
+}
+
+// The call's four words: philox10_rk of (w, ctr, step, slot).
+__device__ __forceinline__ uint4 philox_finish(const PhiloxWord &a, const PhiloxCtr &b, const uint32_t *rk0,
+                                               const uint32_t *rk1)
+{
+    uint4 c = make_uint4(b.x ^ a.y, b.y, a.z ^ b.w2, a.w);
+#pragma unroll
+    for (int round = 3; round < 10; ++round) {
+        const uint64_t p0 = (uint64_t)kPhiloxM0 * c.x;
+        const uint64_t p1 = (uint64_t)kPhiloxM1 * c.z;
+        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ rk0[round], (uint32_t)p1,
+                       (uint32_t)(p0 >> 32) ^ c.w ^ rk1[round], (uint32_t)p0);
+    }
+    return c;
+}
+
+// The four acceptance planes of Philox call n of a site word's stream (words
+// 4n .. 4n + 3, i.e. planes j = 4n - B ..).
+template <int B>
+__device__ __forceinline__ void acceptance_call(const uint4 &z, int n, const uint4 *s_tab, uint32_t c0, uint32_t e1,
+                                                uint32_t &acc, uint32_t &und)
+{
+    const int j0 = 4 * n - B;
+    acceptance_plane(z.x, j0, s_tab, c0, e1, acc, und);
+    acceptance_plane(z.y, j0 + 1, s_tab, c0, e1, acc, und);
+    acceptance_plane(z.z, j0 + 2, s_tab, c0, e1, acc, und);
+    acceptance_plane(z.w, j0 + 3, s_tab, c0, e1, acc, und);
+}
+
 // Acceptance words of Philox calls n = ch_begin .. ch_end - 1 of a site word's
-// stream (words 4n .. 4n + 3, i.e. planes j = 4n - B ..), drawn while a site is
-// undecided: in the whole warp (WARP_VOTE, all lanes must take part) or in this
-// thread's word alone.
+// stream, drawn while a site is undecided: in the whole warp (WARP_VOTE, all
+// lanes must take part) or in this thread's word alone.
 template <int B, bool WARP_VOTE>
-__device__ __forceinline__ void acceptance_calls(int ch_begin, int ch_end, uint32_t w, uint32_t ctr1, uint32_t step,
-                                                 uint32_t slot, const uint32_t *rk0, const uint32_t *rk1,
-                                                 const uint4 *s_tab, uint32_t c0, uint32_t e1, uint32_t &acc,
-                                                 uint32_t &und)
+__device__ __forceinline__ void acceptance_calls(int ch_begin, int ch_end, const PhiloxWord &pw, uint32_t w,
+                                                 uint32_t ctr1, uint32_t step, const uint32_t *rk0,
+                                                 const uint32_t *rk1, const uint4 *s_tab, uint32_t c0, uint32_t e1,
+                                                 uint32_t &acc, uint32_t &und)
 {
 #pragma unroll 1
     for (int ch = ch_begin; ch < ch_end; ++ch) {
         if (WARP_VOTE ? !__any_sync(0xFFFFFFFFu, und) : !und) break;
-        const uint4 z = philox10_rk(make_uint4(w, ctr1 | (uint32_t)ch, step, slot), rk0, rk1);
-        const int j0 = 4 * ch - B;
-        acceptance_plane(z.x, j0, s_tab, c0, e1, acc, und);
-        acceptance_plane(z.y, j0 + 1, s_tab, c0, e1, acc, und);
-        acceptance_plane(z.z, j0 + 2, s_tab, c0, e1, acc, und);
-        acceptance_plane(z.w, j0 + 3, s_tab, c0, e1, acc, und);
+        const uint4 z = philox_finish(pw, philox_ctr(w, ctr1 | (uint32_t)ch, step, rk0, rk1), rk0, rk1);
+        acceptance_call<B>(z, ch, s_tab, c0, e1, acc, und);
+    }
+}
+
+// Proposal planes P = (s + t) mod q of the states in planes W, with t = 1 + u
+// for direction sigma = 0 and q - (1 + u) for sigma = 1 (planes sg, u_p =
+// Z[p + 1], p < B - 1): t = (u ^ sigma) + (q - 1 where sigma) + 1 over B planes,
+// S = s + t, q taken off where S >= q (compared from the lowest plane up).
+// qb / q1b: the bits of q and q - 1 as plane masks.  With q fixed at compile
+// time the masks fold into the three-input logic: 21 operations for q = 10
+// against 28 for s +- (1 + u) with a conditional q added or taken off.
+template <int B, int BP>
+__device__ __forceinline__ void propose(const uint32_t (&W)[BP], const uint32_t *Z, const uint32_t (&qb)[B + 1],
+                                        const uint32_t (&q1b)[B + 1], uint32_t (&P)[BP])
+{
+    const uint32_t sg = Z[0];
+    uint32_t S[B + 1];
+    uint32_t ct = 0xFFFFFFFFu, cs = 0u;
+#pragma unroll
+    for (int p = 0; p < B; ++p) {
+        const uint32_t y = p < B - 1 ? (Z[p + 1] ^ sg) : sg;
+        const uint32_t k = sg & q1b[p];
+        uint32_t t;
+        full_add(y, k, ct, t, ct);
+        full_add(W[p], t, cs, S[p], cs);
+    }
+    S[B] = cs;
+    uint32_t ge = 0xFFFFFFFFu;
+#pragma unroll
+    for (int p = 0; p <= B; ++p) ge = (S[p] & ~qb[p]) | (~(S[p] ^ qb[p]) & ge);
+    uint32_t bw = 0u;
+#pragma unroll
+    for (int p = 0; p < BP; ++p) {
+        if (p < B) {
+            const uint32_t d = ge & qb[p];
+            P[p] = S[p] ^ d ^ bw;
+            bw = (~S[p] & (d | bw)) | (d & bw);
+        } else {
+            P[p] = 0u;
+        }
     }
 }
 
 // Multi-spin-coded sweep body.  B = bits per state (compile time), MODE as
-// for neighbour_planes, Q = q when fixed at compile time (0: q from G).  Each loop step of a thread updates one site word: 32
-// same-colour sites of one row.  The random numbers follow this rule: in
+// for neighbour_planes, Q = q when fixed at compile time (0: q from G).  Each
+// loop step of a thread updates one site word: 32 same-colour sites.  The random numbers follow this rule: in
 // sweep k, colour c, the site word with index w = y WPR + t draws the stream
 // Z_0, Z_1, ... (Z_{4n+i} = word i of the Philox call with counter
 // (w, SWEEP | (2k + c) << 8 | n, step, slot | stream)); the site at bit b takes
 // bit b of each: direction sigma from Z_0, offset u from Z_1..Z_{B-1}, and
 // acceptance bits v_j from Z_{B+j}, most significant first.  Proposal
-// s' = s + (1 + u) mod q (sigma = 0) or s - (1 + u) mod q (sigma = 1) by two
+// s' = s + (1 + u) mod q (sigma = 0) or s - (1 + u) mod q (sigma = 1) by
 // ripple-carry additions over the planes; dE + 4 is the count of eight
 // indicator bits (neighbours equal to s, neighbours different from s'), summed
-// by a carry-save tree; moves with dE > 0 compare v with T[dE] bit by bit, and
-// the warp draws further acceptance words only while some site is undecided.
-template <int B, int MODE, int Q = 0, bool HOIST = false, int QCAP = kQueueCap, bool SPLIT = false>
+// by a carry-save tree; moves with dE > 0 compare v with T[dE] bit by bit.
+//
+// Bound by issue: the logic runs on the ALU pipe (half a warp instruction per
+// clock and scheduler), the Philox products on the FMA-heavy one (a quarter).
+// What is made once per word, per word index or per half sweep is therefore
+// kept out of the 378 instructions per word (409 before the shared Philox
+// rounds, the shorter proposal and the smaller queue entries).  Launches of
+// theta = 10 next to beta_t: 2104 -> 2064 us at q = 10, L = 64, R = 1e5; 9722 ->
+// 9387 at q = 20, L = 256, R = 2e4; 4331 -> 4060 at q = 8, L = 128, R = 5e4; 728 ->
+// 635 at q = 6, L = 32, R = 1e5; 761 -> 656 at q = 8, L = 48, R = 5e4; 3769 -> 3390
+// at q = 3, L = 100, R = 5e4.
+template <int B, int MODE, int Q = 0, int QCAP = kQueueCap, bool LAT = false>
 __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32_t *sw, const uint4 *s_tab,
                                                  uint32_t *qbuf, const uint32_t *rk0, const uint32_t *rk1,
                                                  long long &sE, long long &sE2, long long &sM)
 {
     constexpr int BP = plane_stride(B);
     // the measurement's per-replica counts reuse the queue (at most 16 replicas x (q + 1))
-    static_assert(16 * ((1 << B) + 1) <= queue_words(B, QCAP), "queue too small for the counts");
+    static_assert((LAT ? 8 : 16) * ((1 << B) + 1) <= queue_words(B, QCAP), "queue too small for the counts");
     const int L = MODE == 0 ? 64 : Lrt;
     const int N = L * L;
     const int WPR = MODE == 0 ? 1 : row_words(L);
@@ -447,35 +558,34 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
     }
     __syncthreads();
 
-    // q and 2^(B+1) - q as plane masks, for the reduction mod q
-    uint32_t qm[B + 1], nqm[B + 1];
+    // q and q - 1 as plane masks, for the proposal
+    uint32_t qm[B + 1], q1m[B + 1];
 #pragma unroll
     for (int p = 0; p <= B; ++p) {
         qm[p] = ((q >> p) & 1) ? 0xFFFFFFFFu : 0u;
-        nqm[p] = ((((1 << (B + 1)) - q) >> p) & 1) ? 0xFFFFFFFFu : 0u;
+        q1m[p] = (((q - 1) >> p) & 1) ? 0xFFFFFFFFu : 0u;
     }
     const bool any_full = s_tab[kThresholdFull].x | s_tab[kThresholdFull].y | s_tab[kThresholdFull].z |
                           s_tab[kThresholdFull].w;
-    const int total = nrep * IPC;
 
     // site words still undecided after the first pass wait in qbuf for the second
+    constexpr int EW = queue_entry_words(B) / 4;  // 16-byte vectors per entry
     int *q_count = reinterpret_cast<int *>(qbuf);
-    int *q_item = q_count + 2;
-    uint32_t(*q_mask)[QCAP] = reinterpret_cast<uint32_t(*)[QCAP]>(qbuf + 2 + QCAP);  // acc, und, c0, e1
-    uint32_t(*q_prop)[QCAP] = reinterpret_cast<uint32_t(*)[QCAP]>(qbuf + 2 + 5 * QCAP);
+    uint4 *q_entry = reinterpret_cast<uint4 *>(qbuf + 4);
     if (tid < 2) q_count[tid] = 0;
     __syncthreads();
     int half = 0;
-    // HOIST: when each pass of the block's threads covers whole replicas and
-    // a warp stays within one replica (IPC a multiple of 32 dividing the
-    // threads), a thread keeps one site word index through all passes: its
-    // row, neighbour offsets and counter word are computed once instead of per
-    // word.  (The batched kernel, one function over every body, leaves it out:
-    // a second copy of each first pass doubles its size and build time.)
-    const bool whole_passes = HOIST && IPC % 32 == 0 && (nwarps * 32) % IPC == 0;
-    const int it_fixed = (warp * 32 + lane) % IPC;
-    const int r_first = (warp * 32) / IPC;
-    const int r_step = (nwarps * 32) / IPC;
+    // A thread keeps one site word index through its replicas (several in turn
+    // where a colour has more words than the block threads), so that its row,
+    // neighbour offsets, counter word and the Philox products that follow them
+    // are made once per half sweep.  Threads beyond the last whole replica's
+    // words idle; the launch shapes keep them few.
+    const int threads = (int)blockDim.x;
+    const bool wide = IPC > threads;
+    const int per_pass = wide ? 1 : threads / IPC;
+    const int r_first = wide ? 0 : tid / IPC;
+    const int it_first = r_first < per_pass ? tid - r_first * IPC : IPC;
+    const int it_step = wide ? threads : IPC;
     // replica of a block-wide word index, and row (segment row) of a word
     const uint32_t inv_ipc = div_inverse(IPC);
     const uint32_t inv_row = div_inverse(MODE == 4 ? L >> 4 : WPR);
@@ -486,9 +596,11 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
             const uint32_t ctr1 = DOM_SWEEP | ((uint32_t)(2 * k + c) << 8);
             if (tid == 0) q_count[(half + 1) & 1] = 0;
             int *qc = q_count + (half & 1);
+            constexpr int fc = (B + 3) / 4;  // proposal calls; acceptance calls follow
+            constexpr int kCalls = fc + (LAT ? kLatCalls : kFirstPassCalls);
             // one site word: replica r, word it within the colour (its counter
-            // word w); lanes that are not live run along for the warp votes
-            auto site_word = [&](const int r, const int it, const bool live) {
+            // word w); pc: the calls' shared Philox products
+            auto site_word = [&](const int r, const int it, const PhiloxCtr (&pc)[kCalls]) {
                 const int ii = r * IPC + it;
                 uint32_t *rep = sw + r * RW;
                 uint32_t *own = rep + (c * IPC + it) * BP;
@@ -498,47 +610,22 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
                 const uint32_t vmask =
                     neighbour_planes<B, MODE, BP>(oth, L, IPC, WPR, nb_last, inv_row, it, c, U, D, H, X);
 
-                // proposal: direction sigma = Z_0, offset bits u = Z_1..Z_{B-1}
                 const uint32_t slot = (uint32_t)(first + r) | G.stream_hi;
                 const uint32_t w = (uint32_t)it;
-                uint32_t Z[8];
-                {
-                    const uint4 z = philox10_rk(make_uint4(w, ctr1, (uint32_t)G.step, slot), rk0, rk1);
-                    Z[0] = z.x;
-                    Z[1] = z.y;
-                    Z[2] = z.z;
-                    Z[3] = z.w;
-                }
-                if constexpr (B > 4) {
-                    const uint4 z = philox10_rk(make_uint4(w, ctr1 | 1u, (uint32_t)G.step, slot), rk0, rk1);
-                    Z[4] = z.x;
-                    Z[5] = z.y;
-                    Z[6] = z.z;
-                    Z[7] = z.w;
-                }
-                const uint32_t sg = Z[0];
-                // S = s + 1 + u (sigma = 0) or s - 1 - u (sigma = 1), B + 1 bits
-                uint32_t S[B + 1];
-                uint32_t cy = ~sg;
+                const PhiloxWord pw = philox_word(w, (uint32_t)G.step, slot, rk0, rk1);
+                auto call = [&](int n) { return philox_finish(pw, pc[n], rk0, rk1); };
+                // proposal: direction sigma = Z_0, offset bits u = Z_1..Z_{B-1}
+                uint32_t Z[4 * fc];
 #pragma unroll
-                for (int p = 0; p < B; ++p) {
-                    const uint32_t x = (p < B - 1) ? (Z[p + 1] ^ sg) : sg;
-                    full_add(W[p], x, cy, S[p], cy);
+                for (int n = 0; n < fc; ++n) {
+                    const uint4 z = call(n);
+                    Z[4 * n + 0] = z.x;
+                    Z[4 * n + 1] = z.y;
+                    Z[4 * n + 2] = z.z;
+                    Z[4 * n + 3] = z.w;
                 }
-                S[B] = sg ^ cy;
-                // Tq = S - q (sigma = 0) or S + q (sigma = 1); take Tq where S >= q
-                // (sigma = 0) or S < 0 (sigma = 1)
-                uint32_t Tq[B + 1];
-                uint32_t cz = 0;
-#pragma unroll
-                for (int p = 0; p <= B; ++p) {
-                    const uint32_t yb = (sg & qm[p]) | (~sg & nqm[p]);
-                    full_add(S[p], yb, cz, Tq[p], cz);
-                }
-                const uint32_t take = (sg & S[B]) | (~sg & ~Tq[B]);
                 uint32_t P[BP];
-#pragma unroll
-                for (int p = 0; p < BP; ++p) P[p] = p < B ? ((take & Tq[p]) | (~take & S[p])) : 0u;
+                propose<B, BP>(W, Z, qm, q1m, P);
 
                 // dE + 4 = #(neighbours equal to s) + #(neighbours different from s')
                 const uint32_t a1 = ~differ<B, BP>(W, U), a2 = ~differ<B, BP>(W, D);
@@ -557,85 +644,92 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
                 const uint32_t e1 = c3 | (c1 & c0);                     // dE >= 3
 
                 // acceptance: dE <= 0 always; otherwise v < T[dE], bit by bit
-                uint32_t acc = live ? (vmask & ~pos) : 0u;
-                uint32_t und = live ? pos : 0u;
+                uint32_t acc = vmask & ~pos;
+                uint32_t und = pos;
                 if (any_full) {
                     const uint32_t tj = threshold_bits(s_tab[kThresholdFull], c0, e1);
                     acc |= und & tj;
                     und &= ~tj;
                 }
                 // acceptance bit j is word B + j: the rest of the last proposal call first
-                if constexpr (B % 4 != 0) {
-                    if (__any_sync(0xFFFFFFFFu, und)) {
 #pragma unroll
-                        for (int wi = B; wi < 4 * ((B + 3) / 4); ++wi)
-                            acceptance_plane(Z[wi], wi - B, s_tab, c0, e1, acc, und);
-                    }
-                }
-                constexpr int fc = (B + 3) / 4;
-                acceptance_calls<B, true>(fc, fc + kFirstPassCalls, w, ctr1, (uint32_t)G.step, slot, rk0, rk1, s_tab,
-                                          c0, e1, acc, und);
-                bool queued = false;
+                for (int wi = B; wi < 4 * fc; ++wi) acceptance_plane(Z[wi], wi - B, s_tab, c0, e1, acc, und);
+#pragma unroll
+                for (int n = fc; n < kCalls; ++n) acceptance_call<B>(call(n), n, s_tab, c0, e1, acc, und);
+                if constexpr (LAT) {
+                    acceptance_calls<B, false>(kCalls, fc + 8, pw, w, ctr1, (uint32_t)G.step, rk0, rk1, s_tab, c0, e1,
+                                               acc, und);
+                } else
                 if (und) {
                     const int e = atomicAdd(qc, 1);
                     if (e < QCAP) {
-                        q_item[e] = ii;
-                        q_mask[0][e] = acc;
-                        q_mask[1][e] = und;
-                        q_mask[2][e] = c0;
-                        q_mask[3][e] = e1;
+                        uint4 *dst = q_entry + e * EW;
+                        dst[0] = make_uint4((uint32_t)ii, und, c0, e1);
+                        uint32_t pv[4 * (EW - 1)];
 #pragma unroll
-                        for (int p = 0; p < B; ++p) q_prop[p][e] = P[p];
-                        queued = true;
+                        for (int p = 0; p < 4 * (EW - 1); ++p) pv[p] = p < B ? P[p < BP ? p : 0] : 0u;
+#pragma unroll
+                        for (int h = 0; h < EW - 1; ++h)
+                            dst[1 + h] = make_uint4(pv[4 * h], pv[4 * h + 1], pv[4 * h + 2], pv[4 * h + 3]);
                     } else {
                         // queue full: this thread finishes its word alone (no warp votes)
-                        acceptance_calls<B, false>(fc + kFirstPassCalls, fc + 8, w, ctr1, (uint32_t)G.step, slot, rk0,
-                                                   rk1, s_tab, c0, e1, acc, und);
+                        acceptance_calls<B, false>(kCalls, fc + 8, pw, w, ctr1, (uint32_t)G.step, rk0, rk1, s_tab, c0,
+                                                   e1, acc, und);
                     }
                 }
-                if (live && !queued) {
-                    const uint32_t a = acc & ~und;
+                const uint32_t a = acc & ~und;
 #pragma unroll
-                    for (int p = 0; p < B; ++p) W[p] = (a & P[p]) | (~a & W[p]);
-                    store_planes<BP>(own, W);
-                }
+                for (int p = 0; p < B; ++p) W[p] = (a & P[p]) | (~a & W[p]);
+                store_planes<BP>(own, W);
             };
-            if (HOIST && whole_passes) {
-                for (int r = r_first; r < nrep; r += r_step) site_word(r, it_fixed, true);
-            } else {
-                for (int base = warp * 32; base < total; base += nwarps * 32) {
-                    const int i = base + lane;
-                    const bool live = i < total;
-                    const int ii = live ? i : total - 1;
-                    const int r = replica_of(ii);
-                    site_word(r, ii - r * IPC, live);
+            for (int it = it_first; it < IPC; it += it_step) {
+                PhiloxCtr pc[kCalls];
+#pragma unroll
+                for (int n = 0; n < kCalls; ++n)
+                    pc[n] = philox_ctr((uint32_t)it, ctr1 | (uint32_t)n, (uint32_t)G.step, rk0, rk1);
+                for (int r = r_first; r < nrep; r += per_pass) {
+                    // keeps the row and neighbour arithmetic in the loop: carried
+                    // through it, its registers spill at 64 per thread
+                    int iw = it;
+                    asm volatile("" : "+r"(iw));
+                    site_word(r, iw, pc);
                 }
             }
             __syncthreads();
+            if constexpr (LAT) continue;
             // second pass: the queued site words, 32 to a warp
             const int nq = min(*qc, QCAP);
             for (int base = warp * 32; base < nq; base += nwarps * 32) {
                 const int e = base + lane;
                 const bool live = e < nq;
                 const int ee = live ? e : nq - 1;
-                const int ii = q_item[ee];
+                const uint4 head = q_entry[ee * EW];
+                const int ii = (int)head.x;
                 const int r = replica_of(ii);
                 const int it = ii - r * IPC;
-                uint32_t acc = q_mask[0][ee];
-                uint32_t und = live ? q_mask[1][ee] : 0u;
-                const uint32_t c0 = q_mask[2][ee], e1 = q_mask[3][ee];
+                uint32_t acc = 0u;
+                uint32_t und = live ? head.y : 0u;
+                const uint32_t c0 = head.z, e1 = head.w;
                 const uint32_t slot = (uint32_t)(first + r) | G.stream_hi;
                 const uint32_t w = (uint32_t)it;
-                constexpr int fc = (B + 3) / 4;
-                acceptance_calls<B, true>(fc + kFirstPassCalls, fc + 8, w, ctr1, (uint32_t)G.step, slot, rk0, rk1,
-                                          s_tab, c0, e1, acc, und);
+                const PhiloxWord pw = philox_word(w, (uint32_t)G.step, slot, rk0, rk1);
+                acceptance_calls<B, true>(kCalls, fc + 8, pw, w, ctr1, (uint32_t)G.step, rk0, rk1, s_tab, c0, e1, acc,
+                                          und);
                 if (live) {
                     uint32_t *own = sw + r * RW + (c * IPC + it) * BP;
-                    uint32_t W[BP];
+                    uint32_t W[BP], pv[4 * (EW - 1)];
                     load_planes<BP>(W, own);
+#pragma unroll
+                    for (int h = 0; h < EW - 1; ++h) {
+                        const uint4 a = q_entry[ee * EW + 1 + h];
+                        pv[4 * h + 0] = a.x;
+                        pv[4 * h + 1] = a.y;
+                        pv[4 * h + 2] = a.z;
+                        pv[4 * h + 3] = a.w;
+                    }
                     const uint32_t a = acc & ~und;
 #pragma unroll
-                    for (int p = 0; p < B; ++p) W[p] = (a & q_prop[p][ee]) | (~a & W[p]);
+                    for (int p = 0; p < B; ++p) W[p] = (a & pv[p]) | (~a & W[p]);
                     store_planes<BP>(own, W);
                 }
             }
@@ -643,45 +737,65 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
         }
     }
 
-    if (SPLIT && 2 * nrep <= nwarps) {
-        // measurements of a block holding fewer replicas than twice its warps
-        // (SPLIT: the single-run kernel, whose blocks may hold a few large
-        // lattices): every warp takes a share of each replica's words and the
-        // warps' counts are summed in shared memory (the queue's, idle now),
-        // with one barrier for the group instead of three per count
-        // (nrep <= nwarps / 2 <= 16 replicas x (q + 1) counts fit the queue)
+    // Measurements.  A warp's lanes count their words' agreeing neighbours and
+    // states; a chunk of states is counted per reading of the words and its
+    // warp sums follow one another (one state per reading, each waiting for
+    // its own sum, took 1.7 us per replica and warp at L = 16).
+    auto agreeing = [&](const uint32_t *rep, int me, int stride) {
+        int n = 0;
+        // each bond has one colour-0 end: count equal neighbours of colour-0 sites
+        for (int it = me; it < IPC; it += stride) {
+            uint32_t W[BP], U[BP], D[BP], H[BP], X[BP];
+            load_planes<BP>(W, rep + it * BP);
+            const uint32_t vmask =
+                neighbour_planes<B, MODE, BP>(rep + IPC * BP, L, IPC, WPR, nb_last, inv_row, it, 0, U, D, H, X);
+            n += __popc(vmask & ~differ<B, BP>(W, U)) + __popc(vmask & ~differ<B, BP>(W, D)) +
+                 __popc(vmask & ~differ<B, BP>(W, H)) + __popc(vmask & ~differ<B, BP>(W, X));
+        }
+        return __reduce_add_sync(0xFFFFFFFFu, n);
+    };
+    // emit(s, number of sites in state s) for every state, in every lane
+    auto count_states = [&](const uint32_t *rep, int me, int stride, auto emit) {
+        constexpr int CH = Q == 0 ? 4 : Q % 5 == 0 ? 5 : Q <= 8 ? Q : 8;
+#pragma unroll(Q > 0 ? 32 : 1)
+        for (int s0 = 0; s0 < q; s0 += CH) {
+            int cnt[CH];
+#pragma unroll
+            for (int i = 0; i < CH; ++i) cnt[i] = 0;
+            for (int it = me; it < 2 * IPC; it += stride) {
+                uint32_t W[BP];
+                load_planes<BP>(W, rep + it * BP);
+                const uint32_t vmask = (MODE == 0 || MODE == 3 || MODE == 4)
+                                           ? 0xFFFFFFFFu
+                                           : valid_mask(it - div_by(it, inv_row) * WPR, WPR, nb_last);
+#pragma unroll
+                for (int i = 0; i < CH; ++i) cnt[i] += __popc(vmask & equal_state<B, BP>(W, s0 + i));
+            }
+#pragma unroll
+            for (int i = 0; i < CH; ++i) {
+                const int c = __reduce_add_sync(0xFFFFFFFFu, cnt[i]);
+                if (s0 + i < q) emit(s0 + i, c);
+            }
+        }
+    };
+    if (2 * nrep <= nwarps) {
+        // fewer replicas than half the warps: several warps share each
+        // replica's words and add their counts in shared memory (the queue's,
+        // idle now; nrep <= nwarps / 2 replicas x (q + 1) counts fit it)
         int *s_cnt = reinterpret_cast<int *>(qbuf);
         for (int i = tid; i < nrep * (q + 1); i += blockDim.x) s_cnt[i] = 0;
         __syncthreads();
-        for (int r = 0; r < nrep; ++r) {
+        const int share = nwarps / nrep;  // warps per replica
+        const int r = warp / share;
+        if (r < nrep) {
             const uint32_t *rep = sw + r * RW;
             int *cnt_r = s_cnt + r * (q + 1);
-            int agree = 0;
-            // each bond has one colour-0 end: count equal neighbours of colour-0 sites
-            for (int it = tid; it < IPC; it += blockDim.x) {
-                uint32_t W[BP], U[BP], D[BP], H[BP], X[BP];
-                load_planes<BP>(W, rep + it * BP);
-                const uint32_t vmask =
-                    neighbour_planes<B, MODE, BP>(rep + IPC * BP, L, IPC, WPR, nb_last, inv_row, it, 0, U, D, H, X);
-                agree += __popc(vmask & ~differ<B, BP>(W, U)) + __popc(vmask & ~differ<B, BP>(W, D)) +
-                         __popc(vmask & ~differ<B, BP>(W, H)) + __popc(vmask & ~differ<B, BP>(W, X));
-            }
-            agree = __reduce_add_sync(0xFFFFFFFFu, agree);
-            if (lane == 0 && agree) atomicAdd(cnt_r + q, agree);
-            for (int s = 0; s < q; ++s) {
-                int cnt = 0;
-                for (int it = tid; it < 2 * IPC; it += blockDim.x) {
-                    uint32_t W[BP];
-                    load_planes<BP>(W, rep + it * BP);
-                    const uint32_t vmask =
-                        (MODE == 0 || MODE == 3 || MODE == 4)
-                            ? 0xFFFFFFFFu
-                            : valid_mask(it - div_by(it, inv_row) * WPR, WPR, nb_last);
-                    cnt += __popc(vmask & equal_state<B, BP>(W, s));
-                }
-                cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-                if (lane == 0 && cnt) atomicAdd(cnt_r + s, cnt);
-            }
+            const int me = (warp - r * share) * 32 + lane, stride = share * 32;
+            const int agree = agreeing(rep, me, stride);
+            if (lane == 0) atomicAdd(cnt_r + q, agree);
+            count_states(rep, me, stride, [&](int s, int c) {
+                if (lane == 0) atomicAdd(cnt_r + s, c);
+            });
         }
         __syncthreads();
         // lane 0 of warp r records replica r (lane 0 of each warp carries the sums)
@@ -692,48 +806,13 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
             record_replica(G, first + warp, -cnt_r[q], best, N, sE, sE2, sM);
         }
     } else {
-        // measurements: one warp per replica, or the whole block per replica when
-        // the block holds fewer replicas than warps
-        const bool per_warp = 2 * nrep > nwarps;
-        const int n_owner = per_warp ? nwarps : 1;
-        const int owner = per_warp ? warp : 0;
-        const int stride = per_warp ? 32 : (int)blockDim.x;
-        const int me = per_warp ? lane : tid;
-        for (int r0 = 0; r0 < nrep; r0 += n_owner) {
-            const int r = r0 + owner;
-            const bool have = r < nrep;
-            const uint32_t *rep = sw + (have ? r : 0) * RW;
-            int agree = 0;
-            if (have) {
-                // each bond has one colour-0 end: count equal neighbours of colour-0 sites
-                for (int it = me; it < IPC; it += stride) {
-                    uint32_t W[BP], U[BP], D[BP], H[BP], X[BP];
-                    load_planes<BP>(W, rep + it * BP);
-                    const uint32_t vmask = neighbour_planes<B, MODE, BP>(rep + IPC * BP, L, IPC, WPR, nb_last,
-                                                                         inv_row, it, 0, U, D, H, X);
-                    agree += __popc(vmask & ~differ<B, BP>(W, U)) + __popc(vmask & ~differ<B, BP>(W, D)) +
-                             __popc(vmask & ~differ<B, BP>(W, H)) + __popc(vmask & ~differ<B, BP>(W, X));
-                }
-            }
-            agree = per_warp ? __reduce_add_sync(0xFFFFFFFFu, agree) : block_sum_int(agree);
+        // one warp per replica
+        for (int r = warp; r < nrep; r += nwarps) {
+            const uint32_t *rep = sw + r * RW;
+            const int agree = agreeing(rep, lane, 32);
             int best = 0;
-            for (int s = 0; s < q; ++s) {
-                int cnt = 0;
-                if (have) {
-                    for (int it = me; it < 2 * IPC; it += stride) {
-                        uint32_t W[BP];
-                        load_planes<BP>(W, rep + it * BP);
-                        const uint32_t vmask =
-                            (MODE == 0 || MODE == 3 || MODE == 4)
-                                ? 0xFFFFFFFFu
-                                : valid_mask(it - div_by(it, inv_row) * WPR, WPR, nb_last);
-                        cnt += __popc(vmask & equal_state<B, BP>(W, s));
-                    }
-                }
-                cnt = per_warp ? __reduce_add_sync(0xFFFFFFFFu, cnt) : block_sum_int(cnt);
-                best = max(best, cnt);
-            }
-            if (have && me == 0) record_replica(G, first + r, -agree, best, N, sE, sE2, sM);
+            count_states(rep, lane, 32, [&](int, int c) { best = max(best, c); });
+            if (lane == 0) record_replica(G, first + r, -agree, best, N, sE, sE2, sM);
         }
     }
     group_families(G);
