@@ -239,7 +239,7 @@ class Clocks:
 def _sweep_sources() -> bytes:
     csrc = os.path.join(ROOT, "paper_1704_01888_gb300", "csrc")
     return b"".join(open(os.path.join(csrc, f), "rb").read()
-                    for f in ("pa_sweep.cu", "pa_sweep_body.cuh", "pa_internal.cuh"))
+                    for f in ("pa_sweep.cu", "pa_sweep_kernel.cuh", "pa_sweep_body.cuh", "pa_internal.cuh"))
 
 
 def _sweep_record(w):

@@ -16,8 +16,8 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 LIB = os.path.join(HERE, "libpa_gb300.so")
 # the same library with the kernels' bounds tests compiled in (PA_CHECKED, pa_internal.cuh)
 LIB_CHECKED = os.path.join(HERE, "libpa_gb300_checked.so")
-SOURCES = ["pa_sweep.cu", "pa_resample.cu", "pa_capi.cu", "pa_reweight.cu", "pa_batch.cu", "pa_batch_hi.cu",
-           "pa_noalloc.cu"]
+SOURCES = ["pa_sweep.cu", "pa_sweep_rows.cu", "pa_sweep_lat.cu", "pa_resample.cu", "pa_capi.cu", "pa_reweight.cu",
+           "pa_batch.cu", "pa_batch_hi.cu", "pa_noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -61,32 +61,32 @@ namespace {
 // masks -- else its bits per state, and its row geometry.
 template <int MODE, int PART>
 __device__ __forceinline__ void batch_body(int qv, int B, const dev::Group &G, int L, uint32_t *sw,
-                                           const uint4 *s_tab, uint32_t *q, const BatchArgs &b, long long &sE,
-                                           long long &sE2, long long &sM)
+                                           const uint4 *s_tab, uint32_t *q, const BatchArgs &b,
+                                           unsigned long long *acc)
 {
     if constexpr (PART == 0) {
         switch (qv) {
-        case 5: dev::sweep_group_bits<3, MODE, 5>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); return;
-        case 6: dev::sweep_group_bits<3, MODE, 6>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); return;
-        case 8: dev::sweep_group_bits<3, MODE, 8>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); return;
-        case 10: dev::sweep_group_bits<4, MODE, 10>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); return;
+        case 5: dev::sweep_group_bits<3, MODE, 5>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); return;
+        case 6: dev::sweep_group_bits<3, MODE, 6>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); return;
+        case 8: dev::sweep_group_bits<3, MODE, 8>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); return;
+        case 10: dev::sweep_group_bits<4, MODE, 10>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); return;
         default: break;
         }
         switch (B) {
-        case 1: dev::sweep_group_bits<1, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); break;
-        case 2: dev::sweep_group_bits<2, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); break;
-        case 3: dev::sweep_group_bits<3, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); break;
-        default: dev::sweep_group_bits<4, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); break;
+        case 1: dev::sweep_group_bits<1, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); break;
+        case 2: dev::sweep_group_bits<2, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); break;
+        case 3: dev::sweep_group_bits<3, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); break;
+        default: dev::sweep_group_bits<4, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); break;
         }
     } else {
         if (qv == 20) {
-            dev::sweep_group_bits<5, MODE, 20>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM);
+            dev::sweep_group_bits<5, MODE, 20>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc);
             return;
         }
         switch (B) {
-        case 5: dev::sweep_group_bits<5, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); break;
-        case 6: dev::sweep_group_bits<6, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); break;
-        default: dev::sweep_group_bits<7, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, sE, sE2, sM); break;
+        case 5: dev::sweep_group_bits<5, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); break;
+        case 6: dev::sweep_group_bits<6, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); break;
+        default: dev::sweep_group_bits<7, MODE>(G, L, sw, s_tab, q, b.rk0, b.rk1, acc); break;
         }
     }
 }
@@ -163,20 +163,18 @@ __global__ void __launch_bounds__(1024) k_batch_sweep(const BatchArgs b)
         G.err = &r.st->err;
 #endif
         dev::build_threshold_table(s_tab, sp.thr);
-        long long sE = 0, sE2 = 0, sM = 0;
         uint32_t *sw = reinterpret_cast<uint32_t *>(smem4);
         const int B = state_bits(r.q);
         if (r.L == 64)
-            batch_body<0, PART>(r.q, B, G, 64, sw, s_tab, s_queue, b, sE, sE2, sM);
+            batch_body<0, PART>(r.q, B, G, 64, sw, s_tab, s_queue, b, r.acc);
         else if (r.L % 64 == 0)
-            batch_body<1, PART>(r.q, B, G, r.L, sw, s_tab, s_queue, b, sE, sE2, sM);
+            batch_body<1, PART>(r.q, B, G, r.L, sw, s_tab, s_queue, b, r.acc);
         else if (rows_packed(r.L))
-            batch_body<3, PART>(r.q, B, G, r.L, sw, s_tab, s_queue, b, sE, sE2, sM);
+            batch_body<3, PART>(r.q, B, G, r.L, sw, s_tab, s_queue, b, r.acc);
         else if (rows_banded(r.L))
-            batch_body<4, PART>(r.q, B, G, r.L, sw, s_tab, s_queue, b, sE, sE2, sM);
+            batch_body<4, PART>(r.q, B, G, r.L, sw, s_tab, s_queue, b, r.acc);
         else
-            batch_body<2, PART>(r.q, B, G, r.L, sw, s_tab, s_queue, b, sE, sE2, sM);
-        if ((threadIdx.x & 31) == 0 && (sE | sE2 | sM)) dev::accumulate_totals(r.acc, sE, sE2, sM);
+            batch_body<2, PART>(r.q, B, G, r.L, sw, s_tab, s_queue, b, r.acc);
     }
 }
 

@@ -120,7 +120,9 @@ struct pa_ctx {
     double beta = 0.0;     // inverse temperature of the current population
     bool failed = false;
 
-    int rpb = 1, threads = 32, grid = 1;
+    int rpb = 1, threads = 32, grid = 1;  // replicas a block holds, threads, blocks
+    int group = 1;      // replicas a block takes at a time (at most rpb)
+    bool lat = false;   // the latency kernel
 
     // A population spread over several GPUs (pa_shard_init): this context
     // holds the global slots [slot0, slot0 + R_i(local)) of one population of
@@ -291,27 +293,129 @@ constexpr size_t kStageObs = 256;
 constexpr size_t kStageHist = 512;
 static_assert(sizeof(pa::DevState) <= kStageObs && sizeof(pa_obs) <= kStageHist - kStageObs, "staging layout");
 
+// Warp passes of one block per half sweep (a warp with any live lane counts)
+// and passes of its threads, for rpb replicas of `units` site words per colour.
+struct BlockWork {
+    long long warps, passes;
+};
+BlockWork block_work(int rpb, long long units, int threads)
+{
+    if (units > threads) return {rpb * ((units + 31) / 32), rpb * ((units + threads - 1) / threads)};
+    const long long per_pass = threads / units, full = rpb / per_pass, rest = rpb % per_pass;
+    return {full * ((per_pass * units + 31) / 32) + (rest * units + 31) / 32, full + (rest > 0)};
+}
+
+// Cost of one half sweep, in about a microsecond, of a launch that keeps k
+// blocks on an SM.  It is bound by issue (proportional to the SM's warp
+// passes, a little worse with fewer than 32 warps resident) or, with few
+// warps, by the latency of one word's chain per pass; to it come the barriers
+// and the queue pass, less of them visible with more independent blocks, and
+// the share of the step's load, measurement (per replica of a warp) and store.
+// Fitted to launches of theta = 10 at q = 10, L = 64: 3.6, 5.5 and 11.6 us per
+// half sweep for 28, 56 and 136 warp passes per SM.  The latency kernel
+// (lat) takes 2.2 us for 14 and 1.3 us for 2 where the other takes 2.3 and 1.6.
+double half_sweep_cost(bool lat, int k, int rpb, long long units, int threads)
+{
+    const BlockWork w = block_work(rpb, units, threads);
+    const double resident = k * threads / 32.0, measured = 0.03 * rpb / (threads / 32.0);
+    if (lat) return 1.0 + measured + std::max(0.078 * (double)(k * w.warps), 0.4 * (double)w.passes);
+    const double slack = 1.0 + 0.2 * std::max(0.0, 32.0 - resident) / 32.0;
+    return 0.9 + 1.0 / k + measured + std::max(0.074 * slack * (double)(k * w.warps), 0.6 * (double)w.passes);
+}
+
+// The automatic launch shape: blocks per SM k, rounds m and threads with the
+// least m x half_sweep_cost, where the k m blocks per SM share the population
+// evenly (a few replicas more than R are planned for: the copy numbers
+// spread by at most about sqrt(R)).  Equal shares matter most for small and
+// middling populations: 10^4 replicas of L = 32 in 625 groups on 608 blocks
+// took two rounds for 1.03, and 1000 replicas one to a block filled some SMs
+// and left others empty.  The latency kernel (no queue and one barrier per
+// half sweep, three acceptance calls drawn together, up to 128 registers and 16
+// warps per SM) serves the launches whose threads have one site word each.
+// Ties go to more, smaller blocks.
+bool plan_launch(pa_ctx *c)
+{
+    const long long units = pa::colour_words(c->cfg.L);
+    const size_t RB = pa::replica_bytes(c->cfg.q, c->cfg.L);
+    const long long R = c->R_fill + 2 * (long long)std::ceil(std::sqrt((double)c->R_fill));
+    constexpr size_t kSmem = 227 * 1024, kSmemBlock = 16 * 1024;  // per SM; a block's tables and queue
+    double best = 1e300;
+    int b_rpb = 0, b_threads = 0, b_k = 0;
+    bool b_lat = false;
+    for (int lat = 1; lat >= 0; --lat) {
+        const int max_threads = lat ? 512 : 1024;  // per SM: 128 or 64 registers a thread
+        for (int k = 1; k <= 16; ++k) {
+            const size_t room =
+                kSmem / k < kSmemBlock ? 0 : std::min(kSmem / k - kSmemBlock, (size_t)pa::kMaxLatticeBytes);
+            const long long fit = (long long)(room / RB);
+            if (fit < 1) break;
+            const long long slots = (long long)c->sms * k;
+            const long long m0 = (R + slots * fit - 1) / (slots * fit);
+            if (lat && m0 > 1) continue;
+            for (long long m = m0; m < m0 + (lat ? 1 : 4); ++m) {
+                const int rpb = (int)((R + slots * m - 1) / (slots * m));
+                const int top = max_threads / k / 32 * 32;
+                for (long long p = 1; p <= 8; ++p) {
+                    long long t = units <= top ? (rpb + p - 1) / p * units : (units + p - 1) / p;
+                    if (t > top) t = units <= top ? top / units * units : top;
+                    t = std::min<long long>((t + 31) / 32 * 32, top);
+                    if (t < 32 || (lat && block_work(rpb, units, (int)t).passes > 1)) continue;
+                    const double cost = (double)m * half_sweep_cost(lat != 0, k, rpb, units, (int)t);
+                    if (cost < best * 0.995 || (cost <= best * 1.005 && k > b_k && t >= 256)) {
+                        best = std::min(best, cost);
+                        b_rpb = rpb;
+                        b_threads = (int)t;
+                        b_k = k;
+                        b_lat = lat != 0;
+                    }
+                }
+            }
+        }
+    }
+    if (!b_k || pa::sweep_max_blocks_per_sm(c->cfg.q, c->cfg.L, b_rpb, b_threads, b_lat) < b_k) return false;
+    c->rpb = c->group = b_rpb;
+    c->threads = b_threads;
+    c->lat = b_lat;
+    c->grid = (int)std::min((long long)c->sms * b_k, (R + b_rpb - 1) / b_rpb);
+    return true;
+}
+
+// L = 256 and 128 (1024 or 256 site words per colour) with at most five planes:
+// one block of 1024 threads per SM holding as many lattices as fit in whole
+// passes, each thread on one site word index.  At L = 256 five q = 20 lattices
+// a block measure what two blocks of two and 512 threads do (1401 against
+// 1413 attempts/ns); at L = 128 a population of eight rounds or more is left
+// to plan_launch (two blocks of 512: 2108 against 2018).  A block then takes
+// an equal share per round rather than all that it holds (R = 10^4, L = 128:
+// 22 of 24 lattices, 812 us against 871 per launch of theta = 10).
+bool wide_launch(pa_ctx *c)
+{
+    const long long units = pa::colour_words(c->cfg.L);
+    const size_t RB = pa::replica_bytes(c->cfg.q, c->cfg.L);
+    if ((units != 1024 && units != 256) || pa::state_bits(c->cfg.q) > 5 || c->R_fill / (4 * c->sms) < 4) return false;
+    const long long R = c->R_fill + 2 * (long long)std::ceil(std::sqrt((double)c->R_fill));
+    const int per_pass = (int)(1024 / units);
+    const int rpb = (int)((size_t)pa::kMaxLatticeBytes / RB) / per_pass * per_pass;
+    const long long rounds = (R + (long long)c->sms * rpb - 1) / ((long long)c->sms * rpb);
+    if (units == 256 && rounds > 8) return false;
+    if (pa::sweep_max_blocks_per_sm(c->cfg.q, c->cfg.L, rpb, 1024, false) < 1) return false;
+    c->rpb = rpb;
+    c->group = (int)std::min<long long>(rpb, (R + c->sms * rounds - 1) / (c->sms * rounds));
+    c->threads = 1024;
+    c->lat = false;
+    c->grid = (int)std::min<long long>(c->sms, (R + c->group - 1) / c->group);
+    return true;
+}
+
 pa_status choose_launch(pa_ctx *c, int rpb_req, int threads_req)
 {
     const int L = c->cfg.L;
     const size_t RB = pa::replica_bytes(c->cfg.q, L);
+    if (rpb_req <= 0 && threads_req <= 0 && (wide_launch(c) || plan_launch(c))) return PA_OK;
     // work items per replica and half sweep: the site words of one colour
     const long long units = pa::colour_words(L);
     int rpb = rpb_req;
     int threads = threads_req;
-    if (rpb <= 0 && threads <= 0 && (units == 1024 || units == 256) && pa::state_bits(c->cfg.q) <= 5 &&
-        c->R_fill / (4 * c->sms) >= 4) {
-        // 1024 or 256 site words per colour (L = 256, 128): blocks of 1024
-        // threads, each keeping one site word index through all passes, with
-        // as many lattices as fit in whole passes (L = 256, q = 20: five, 1439
-        // against 1339 attempts/ns with two lattices and 512 threads; q = 6:
-        // 1855 against 1731; q = 10 even.  L = 128: q = 20 1411 against 1243,
-        // q = 8 1952 against 1919, q = 5 1857 against 1829, q = 10 even.  With
-        // six or seven planes the 1024-thread blocks are slower)
-        const int per_pass = (int)(1024 / units);
-        rpb = (int)((size_t)pa::kMaxLatticeBytes / RB) / per_pass * per_pass;
-        threads = 1024;
-    }
     if (rpb <= 0) {
         // 96 KB of lattices per block: two blocks of 512 threads per SM
         int rpb_mem = (int)(98304 / RB);
@@ -319,36 +423,27 @@ pa_status choose_launch(pa_ctx *c, int rpb_req, int threads_req)
         int rpb_fill = c->R_fill / (4 * c->sms);
         if (rpb_fill < 1) rpb_fill = 1;
         rpb = rpb_mem < rpb_fill ? rpb_mem : rpb_fill;
-        // a group spanning several passes of 512 threads over its site words
-        // fills each pass: q = 10, L = 64 takes 48 replicas (6 words per
-        // thread), not 44 (5.5)
-        const long long per_pass = 512 / units;
-        if (per_pass >= 1 && rpb > per_pass) rpb = (int)(rpb / per_pass * per_pass);
-        // at least one warp of work items per block
-        const int rpb_warp = (int)((32 + units - 1) / units);
-        if (rpb < rpb_warp) rpb = rpb_warp < rpb_mem ? rpb_warp : rpb_mem;
     }
     if ((size_t)rpb * RB > (size_t)pa::kMaxLatticeBytes) return rpb == 1 ? PA_ERR_TOO_LARGE : PA_ERR_INVALID;
     if (threads <= 0) {
-        // one thread per site word, at most 512; a block that holds a single
-        // large replica takes about four words per thread instead (measured
-        // best at q = 20, L = 256: fewer words per thread leave the barriers
-        // and the queue pass of each half sweep poorly amortised)
+        // one thread per site word, at most 512
         const long long work = (long long)rpb * units;
-        const long long per_thread = rpb == 1 ? 4 : 1;
-        threads = (int)(((work + per_thread - 1) / per_thread + 31) / 32 * 32);
-        if (threads > 512) threads = 512;
-        if (threads < 32) threads = 32;
+        threads = (int)std::min<long long>((work + 31) / 32 * 32, 512);
     }
     if (threads % 32 != 0 || threads > 1024) return PA_ERR_INVALID;
-    const int per_sm = pa::sweep_max_blocks_per_sm(c->cfg.q, L, rpb, threads);
-    if (per_sm <= 0) return PA_ERR_INVALID;
     const long long groups = ((long long)c->R_cap + rpb - 1) / rpb;
-    long long grid = (long long)per_sm * c->sms;
-    if (grid > groups) grid = groups;
-    c->rpb = rpb;
+    // the latency kernel where its blocks are all resident at once
+    bool lat = threads <= 512 && groups * threads <= 512LL * c->sms;
+    int per_sm = pa::sweep_max_blocks_per_sm(c->cfg.q, L, rpb, threads, lat);
+    if (per_sm <= 0 && lat) {
+        lat = false;
+        per_sm = pa::sweep_max_blocks_per_sm(c->cfg.q, L, rpb, threads, lat);
+    }
+    if (per_sm <= 0) return PA_ERR_INVALID;
+    c->rpb = c->group = rpb;
     c->threads = threads;
-    c->grid = (int)grid;
+    c->lat = lat;
+    c->grid = (int)std::min((long long)per_sm * c->sms, groups);
     return PA_OK;
 }
 
@@ -377,14 +472,15 @@ pa::SweepArgs sweep_args(pa_ctx *c, double beta, int theta, int step, int gather
     a.L = c->cfg.L;
     a.theta = theta;
     a.step = step;
-    a.rpb = c->rpb;
+    a.rpb = c->group;
+    a.lat = c->lat;
     a.gather = gather;
     a.stream_hi = (uint32_t)c->cfg.stream << 24;
     a.slot0 = (uint32_t)c->slot0;
     // few groups per block: hand them out from a counter, so that the blocks
     // end together; with many, equal shares (their ends even out)
     const long long R_est = c->R_fill > 0 ? c->R_fill : c->cfg.R;
-    a.work = R_est < 16LL * c->rpb * c->grid ? c->work : nullptr;
+    a.work = R_est < 16LL * c->group * c->grid ? c->work : nullptr;
     return a;
 }
 

@@ -115,6 +115,7 @@ struct SweepArgs {
     int32_t gather;            // 1: read parents from buf[parity], write buf[parity^1]
     uint32_t stream_hi;        // stream number << 24 (top byte of the slot counter word)
     uint32_t slot0;            // global slot of local slot 0 (0 unless the population spans GPUs)
+    int32_t lat;               // 1: the kernel for launches too small to fill the SMs
     int32_t *work;             // next replica group to hand out (zeroed before each launch), or
                                // null: each block takes an equal share
 };
@@ -122,7 +123,7 @@ struct SweepArgs {
 // Launchers (pa_sweep.cu)
 cudaError_t launch_sweep(const SweepArgs &a, int threads, int grid, cudaStream_t s);
 size_t sweep_smem_bytes(int q, int L, int rpb);
-int sweep_max_blocks_per_sm(int q, int L, int rpb, int threads);
+int sweep_max_blocks_per_sm(int q, int L, int rpb, int threads, bool lat);
 
 // Launchers (pa_resample.cu)
 // slot0: global slot of local slot 0 (random keys and family ids follow it).

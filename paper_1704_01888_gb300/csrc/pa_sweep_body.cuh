@@ -88,6 +88,13 @@ __device__ __forceinline__ uint32_t equal_state(const uint32_t (&a)[BP], int s)
     return ~d;
 }
 
+__device__ __forceinline__ void accumulate_totals(unsigned long long *acc, long long sE, long long sE2, long long sM)
+{
+    atomicAdd(acc + 0, (unsigned long long)sE);
+    atomicAdd(acc + 1, (unsigned long long)sE2);
+    atomicAdd(acc + 2, (unsigned long long)sM);
+}
+
 // Division by a divisor d fixed for a replica group (d < 2^15) of x < 2^16,
 // without a division instruction sequence per use: with inv = ceil(2^31 / d)
 // = (2^31 + e) / d, 0 <= e < d, floor(x inv / 2^31) = floor(x / d) because
@@ -520,7 +527,7 @@ __device__ __forceinline__ void propose(const uint32_t (&W)[BP], const uint32_t 
 template <int B, int MODE, int Q = 0, int QCAP = kQueueCap, bool LAT = false>
 __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32_t *sw, const uint4 *s_tab,
                                                  uint32_t *qbuf, const uint32_t *rk0, const uint32_t *rk1,
-                                                 long long &sE, long long &sE2, long long &sM)
+                                                 unsigned long long *totals)
 {
     constexpr int BP = plane_stride(B);
     // the measurement's per-replica counts reuse the queue (at most 16 replicas x (q + 1))
@@ -737,6 +744,9 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
         }
     }
 
+    // sums of the replicas this warp records (lane 0), added up per group: kept
+    // over the groups they would take six registers through the sweeps
+    long long sE = 0, sE2 = 0, sM = 0;
     // Measurements.  A warp's lanes count their words' agreeing neighbours and
     // states; a chunk of states is counted per reading of the words and its
     // warp sums follow one another (one state per reading, each waiting for
@@ -815,6 +825,7 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
             if (lane == 0) record_replica(G, first + r, -agree, best, N, sE, sE2, sM);
         }
     }
+    if (lane == 0 && (sE | sE2 | sM)) accumulate_totals(totals, sE, sE2, sM);
     group_families(G);
     __syncthreads();
     if (G.write_back) {
@@ -825,13 +836,6 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
         }
     }
     __syncthreads();
-}
-
-__device__ __forceinline__ void accumulate_totals(unsigned long long *acc, long long sE, long long sE2, long long sM)
-{
-    atomicAdd(acc + 0, (unsigned long long)sE);
-    atomicAdd(acc + 1, (unsigned long long)sE2);
-    atomicAdd(acc + 2, (unsigned long long)sM);
 }
 
 }  // namespace dev
