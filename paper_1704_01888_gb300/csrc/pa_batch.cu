@@ -53,19 +53,20 @@ __global__ void k_batch_init(const BatchArgs b)
     }
 }
 
-__global__ void __launch_bounds__(kB) k_batch_weights(const BatchArgs b)
+// One cluster of kBatchCluster blocks per run.
+constexpr int kBatchCluster = 4;
+__global__ void __launch_bounds__(dev::kWeightsThreads) k_batch_weights(const BatchArgs b)
 {
-    __shared__ unsigned long long s_acc[dev::kSumLimbs];
-    __shared__ long long s_l[32];
-    const int m = blockIdx.x;
+    __shared__ dev::WeightsShared sh;
+    const int m = blockIdx.x / kBatchCluster;
     const int i = *b.step_counter;
     const StepDev sp = b.steps[(size_t)i * b.M + m];
     if (!sp.active) return;
     const RunDev &r = b.runs[m];
-    dev::weights_body(r.hist, r.nbins, sp.dbeta, sp.wtab, r.st, s_acc, s_l);
+    dev::weights_body(r.hist, r.nbins, sp.dbeta, sp.wtab, r.st, sh);
 }
 
-__global__ void __launch_bounds__(kB) k_batch_counts(const BatchArgs b)
+__global__ void __launch_bounds__(kChunk) k_batch_counts(const BatchArgs b)
 {
     __shared__ int s_i[32];
     const int m = run_of_chunk(b.runs, b.M, blockIdx.x);
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(kB) k_batch_counts(const BatchArgs b)
                      r.counts, r.local_off, r.blocksum, r.st, s_i);
 }
 
-__global__ void __launch_bounds__(kB) k_batch_scatter(const BatchArgs b)
+__global__ void __launch_bounds__(kChunk) k_batch_scatter(const BatchArgs b)
 {
     __shared__ long long s_l[32];
     const int m = run_of_chunk(b.runs, b.M, blockIdx.x);
@@ -260,9 +261,10 @@ pa_status enqueue_start(pa_batch *b)
 // Enqueues one temperature step (the six launches).
 pa_status enqueue_step(pa_batch *b, cudaStream_t s)
 {
-    pa::k_batch_weights<<<b->M, pa::kB, 0, s>>>(b->args);
-    pa::k_batch_counts<<<b->args.total_chunks, pa::kB, 0, s>>>(b->args);
-    pa::k_batch_scatter<<<b->args.total_chunks, pa::kB, 0, s>>>(b->args);
+    PB_CK(pa::launch_clusters(pa::k_batch_weights, pa::kBatchCluster, pa::kBatchCluster * b->M,
+                              pa::dev::kWeightsThreads, 0, s, b->args));
+    pa::k_batch_counts<<<b->args.total_chunks, pa::kChunk, 0, s>>>(b->args);
+    pa::k_batch_scatter<<<b->args.total_chunks, pa::kChunk, 0, s>>>(b->args);
     launch_sweeps(b, b->args, s);
     pa::k_batch_finalize<<<b->M, pa::kB, 0, s>>>(b->args);
     pa::k_batch_advance<<<1, 1, 0, s>>>(b->counter_d);
@@ -406,7 +408,7 @@ pa_status pa_batch_create(const pa_run_desc *runs, int32_t M, void *cuda_stream,
         r.K = d.K;
         r.ground = g.init_mode == PA_INIT_GROUND;
         r.stream_hi = (uint32_t)g.stream << 24;
-        const int nc = std::max((r.R_cap + pa::kB - 1) / pa::kB, (r.nbins + pa::kB - 1) / pa::kB);
+        const int nc = (r.R_cap + pa::kChunk - 1) / pa::kChunk;
         r.chunk0 = chunk0;
         r.nchunks = nc;
         chunk0 += nc;

@@ -13,6 +13,7 @@
 namespace pa {
 
 constexpr int kB = 1024;
+constexpr int kChunk = 256;  // replicas per block of the copy-number and scatter kernels
 constexpr int kMaxRuns = 1024;
 
 struct RunDev {

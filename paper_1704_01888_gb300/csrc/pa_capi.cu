@@ -614,7 +614,7 @@ pa_status ctx_create(const pa_config &g, void *cuda_stream, pa_ctx **out, int ra
     // a shard's children (parent map, run scan) can number up to the whole
     // population's capacity, its own replicas only up to its share
     const int R_child = (int)R_cap;
-    const int nb = (R_child + 1023) / 1024;
+    const int nb = std::max((R_child + 1023) / 1024, pa::resample_blocks(R_child));
     if ((s = dev_alloc(&c->spins[0], spin_bytes)) || (s = dev_alloc(&c->spins[1], spin_bytes)) ||
         (s = dev_alloc(&c->E, c->R_cap)) || (s = dev_alloc(&c->Mt, c->R_cap)) ||
         (s = dev_alloc(&c->hist, c->nbins)) || (s = dev_alloc(&c->counts, c->R_cap)) ||

@@ -125,6 +125,13 @@ cudaError_t launch_sweep(const SweepArgs &a, int threads, int grid, cudaStream_t
 size_t sweep_smem_bytes(int q, int L, int rpb);
 int sweep_max_blocks_per_sm(int q, int L, int rpb, int threads, bool lat);
 
+// Replicas per block of the copy-number and scatter kernels: 128, so that even
+// small populations' FP64 work spreads over the SMs (10^4 replicas in blocks of
+// 1024: 8.0 us, Poisson 120 us), up to the capacity at which every scatter
+// block's sum over the blocks before it would outweigh that.
+__host__ __device__ constexpr int resample_chunk(int R_cap) { return R_cap <= (1 << 17) ? 128 : R_cap <= (1 << 20) ? 256 : 1024; }
+inline int resample_blocks(int R_cap) { return (R_cap + resample_chunk(R_cap) - 1) / resample_chunk(R_cap); }
+
 // Launchers (pa_resample.cu)
 // slot0: global slot of local slot 0 (random keys and family ids follow it).
 cudaError_t launch_init(uint32_t *spins, int32_t *anc, int q, int L, int R, uint32_t k0, uint32_t k1,

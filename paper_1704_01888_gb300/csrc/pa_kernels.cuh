@@ -11,6 +11,7 @@
 #include <climits>
 #include <type_traits>
 
+#include "pa_cluster.cuh"
 #include "pa_sweep_body.cuh"
 
 namespace pa {
@@ -266,23 +267,16 @@ __device__ __forceinline__ int exact_term(uint32_t h, double w, uint32_t (&c)[4]
 // Adds the terms of the occupied bins among k_begin .. k_end - 1 to the
 // shared limbs.  Consecutive bins have weights within a few binades of one
 // another, so a thread sums its terms in five register limbs (li - 1 .. li +
-// 3 of the first term) and adds them to the shared array only when a term
-// falls outside them: a handful of shared atomics per thread instead of four
-// per term.
+// 3 of the first term) and adds them to the shared array itself only when a
+// term falls outside them; at the end the lanes of a warp whose limbs start at
+// the same place add theirs up by shuffles and one lane adds the sums (64-bit
+// shared atomics on the same few limbs are compare-and-swap loops).  Every
+// thread of the block takes part.
 __device__ __forceinline__ void exact_add_range(unsigned long long *acc, const int32_t *hist, const double *wtab,
                                                 int kref, int k_begin, int k_end)
 {
-    unsigned long long w0 = 0ull, w1 = 0ull, w2 = 0ull, w3 = 0ull, w4 = 0ull;
+    unsigned long long w[5] = {0ull, 0ull, 0ull, 0ull, 0ull};
     int base = -2;
-    auto flush = [&]() {
-        if (base < 0) return;
-        if (w0) atomicAdd(acc + base, w0);
-        if (w1) atomicAdd(acc + base + 1, w1);
-        if (w2) atomicAdd(acc + base + 2, w2);
-        if (w3) atomicAdd(acc + base + 3, w3);
-        if (w4) atomicAdd(acc + base + 4, w4);
-        w0 = w1 = w2 = w3 = w4 = 0ull;
-    };
     // four bins at a time: their loads issue together
     for (int k0 = k_begin; k0 < k_end; k0 += 4) {
         int h[4];
@@ -300,23 +294,35 @@ __device__ __forceinline__ void exact_add_range(unsigned long long *acc, const i
             uint32_t c[4];
             const int li = exact_term((uint32_t)h[i], wk[i], c);
             if (li < base || li > base + 1) {
-                flush();
+                if (base >= 0) {
+#pragma unroll
+                    for (int l = 0; l < 5; ++l) {
+                        if (w[l]) atomicAdd(acc + base + l, w[l]);
+                        w[l] = 0ull;
+                    }
+                }
                 base = li > 0 ? li - 1 : 0;
             }
-            if (li == base) {
-                w0 += c[0];
-                w1 += c[1];
-                w2 += c[2];
-                w3 += c[3];
-            } else {
-                w1 += c[0];
-                w2 += c[1];
-                w3 += c[2];
-                w4 += c[3];
-            }
+            const bool up = li != base;
+            w[0] += up ? 0u : c[0];
+            w[1] += up ? c[0] : c[1];
+            w[2] += up ? c[1] : c[2];
+            w[3] += up ? c[2] : c[3];
+            w[4] += up ? c[3] : 0u;
         }
     }
-    flush();
+    const int lane = threadIdx.x & 31;
+    unsigned pending = __ballot_sync(0xFFFFFFFFu, base >= 0);
+    while (pending) {
+        const int at = __shfl_sync(0xFFFFFFFFu, base, __ffs(pending) - 1);
+        const bool mine = base == at;
+#pragma unroll
+        for (int l = 0; l < 5; ++l) {
+            const unsigned long long sum = warp_sum(mine ? w[l] : 0ull);
+            if (lane == 0 && sum) atomicAdd(acc + at + l, sum);
+        }
+        pending &= ~__ballot_sync(0xFFFFFFFFu, mine);
+    }
 }
 
 // Bits lowpos .. lowpos + 63 of normalised 32-bit limbs (lowpos >= 0).
@@ -332,21 +338,22 @@ __device__ __forceinline__ unsigned long long limb_bits64(const unsigned long lo
 // double (one thread; the value must be at least 1, i.e. bit 1074 or above).
 __device__ __forceinline__ double exact_round(unsigned long long *acc)
 {
-    unsigned long long carry = 0ull;
+    unsigned long long carry = 0ull, nonzero = 0ull;  // bit i: limb i is not zero
+#pragma unroll
     for (int i = 0; i < kSumLimbs; ++i) {
         const unsigned long long v = acc[i] + carry;
         acc[i] = v & 0xFFFFFFFFull;
         carry = v >> 32;
+        nonzero |= (unsigned long long)((uint32_t)v != 0u) << i;
     }
-    int t = kSumLimbs - 1;
-    while (t > 0 && acc[t] == 0ull) --t;
+    if (!nonzero) return 0.0;
+    const int t = 63 - __clzll((long long)nonzero);
     int p = 32 * t + 31 - __clz((uint32_t)acc[t]);  // top bit
     const unsigned long long x = limb_bits64(acc, p - 63);  // bit 63 = top bit
     unsigned long long mant = x >> 11;
     const bool round = (x >> 10) & 1ull;
-    bool sticky = (x & 0x3FFull) != 0ull;
     const int low = p - 63;  // bits below it
-    for (int i = 0; i < (low >> 5) && !sticky; ++i) sticky = acc[i] != 0ull;
+    bool sticky = (x & 0x3FFull) != 0ull || (nonzero & ((1ull << (low >> 5)) - 1ull)) != 0ull;
     if (!sticky && (low & 31)) sticky = (acc[low >> 5] & ((1ull << (low & 31)) - 1ull)) != 0ull;
     if (round && (sticky || (mant & 1ull))) mant += 1ull;
     if (mant >> 53) {
@@ -357,55 +364,60 @@ __device__ __forceinline__ double exact_round(unsigned long long *acc)
     return __longlong_as_double((long long)(((unsigned long long)(p - 51) << 52) | (mant & 0xFFFFFFFFFFFFFull)));
 }
 
-// One block: reference bin, S (exact sum of h_k w_k, weights from the host
+// One cluster: reference bin, S (exact sum of h_k w_k, weights from the host
 // table wtab by distance |k - k_ref|) and ln Q of the pending resample.
+// Latency bound: a reading of the histogram for its occupied range, one of
+// that range with its weights, and a serial rounding.  The blocks share the
+// bins and the first adds up their limbs (in one block: 10, 25 and 97 us with
+// 2049, 32769 and 131073 bins).
 // R_prev_all: the population size R_{i-1} when the histogram covers several
 // GPUs' replicas (0: this GPU's own, st->pop).
+struct WeightsShared {
+    unsigned long long acc[kSumLimbs], sum[kSumLimbs];
+    int sc[64], ext[2];
+};
+constexpr int kWeightsThreads = 512;
 __device__ __forceinline__ void weights_body(const int32_t *hist, int nbins, double dbeta, const double *wtab,
-                                             DevState *st, unsigned long long *s_acc, long long *s_l,
-                                             int R_prev_all = 0)
+                                             DevState *st, WeightsShared &sh, int R_prev_all = 0)
 {
-    if (st->err) return;
-    const int tid = threadIdx.x;
-    // reference bin: lowest occupied for dbeta >= 0, highest for dbeta < 0
-    long long best = dbeta >= 0.0 ? (long long)INT_MAX : -1;
-#pragma unroll 4
-    for (int k = tid; k < nbins; k += blockDim.x) {
-        if (hist[k] > 0) best = dbeta >= 0.0 ? min(best, (long long)k) : max(best, (long long)k);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const long long other = __shfl_down_sync(0xFFFFFFFFu, best, o);
-        best = dbeta >= 0.0 ? min(best, other) : max(best, other);
-    }
-    const int lane = tid & 31, warp = tid >> 5;
-    if (lane == 0) s_l[warp] = best;
-    for (int i = tid; i < kSumLimbs; i += blockDim.x) s_acc[i] = 0ull;
-    __syncthreads();
-    if (warp == 0) {
-        long long v = (lane < (int)(blockDim.x >> 5)) ? s_l[lane] : (dbeta >= 0.0 ? (long long)INT_MAX : -1);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const long long other = __shfl_down_sync(0xFFFFFFFFu, v, o);
-            v = dbeta >= 0.0 ? min(v, other) : max(v, other);
+    if (st->err) return;  // the same in every block
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), c = (int)cl.block_rank(), tid = threadIdx.x, n = blockDim.x;
+    for (int i = tid; i < kSumLimbs; i += n) sh.acc[i] = 0ull;
+    int lo = INT_MAX, hi = -1;
+#pragma unroll 8
+    for (int k = c * n + tid; k < nbins; k += C * n) {
+        if (hist[k] > 0) {
+            lo = min(lo, k);
+            hi = max(hi, k);
         }
-        if (lane == 0) s_l[0] = v;
     }
-    __syncthreads();
-    const int kref = (int)s_l[0];
-    const int per = (nbins + (int)blockDim.x - 1) / (int)blockDim.x;  // a contiguous range of bins per thread
-    exact_add_range(s_acc, hist, wtab, kref, min(nbins, tid * per), min(nbins, (tid + 1) * per));
-    __syncthreads();
-    if (tid == 0) {
-        const double S = exact_round(s_acc);
-        const int E_ref = kref - (nbins - 1);
-        st->S = S;
-        st->E_ref = E_ref;
-        st->ties = 0;
-        const int R_prev = R_prev_all > 0 ? R_prev_all : st->pop;
-        st->lnQ = __dadd_rn(__dmul_rn(-dbeta, (double)E_ref), log(S / (double)R_prev));
+    cluster_extremes(cl, lo, hi, sh.sc, sh.ext);
+    // reference bin: lowest occupied for dbeta >= 0, highest for dbeta < 0
+    const int kref = dbeta >= 0.0 ? lo : hi;
+    const long long range = lo <= hi ? (long long)hi - lo + 1 : 0;
+    const int k0 = lo + (int)(range * c / C), k1 = lo + (int)(range * (c + 1) / C);
+    const int per = (k1 - k0 + n - 1) / n;  // a contiguous range of bins per thread
+    exact_add_range(sh.acc, hist, wtab, kref, min(k1, k0 + tid * per), min(k1, k0 + (tid + 1) * per));
+    cl.sync();
+    if (c == 0) {
+        if (tid < kSumLimbs) {
+            unsigned long long s = 0ull;
+            for (int r = 0; r < C; ++r) s += cl.map_shared_rank(sh.acc, r)[tid];
+            sh.sum[tid] = s;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            const double S = exact_round(sh.sum);
+            const int E_ref = kref - (nbins - 1);
+            st->S = S;
+            st->E_ref = E_ref;
+            st->ties = 0;
+            const int R_prev = R_prev_all > 0 ? R_prev_all : st->pop;
+            st->lnQ = __dadd_rn(__dmul_rn(-dbeta, (double)E_ref), log(S / (double)R_prev));
+        }
     }
-    __syncthreads();
+    cl.sync();  // the blocks' limbs stay until the first has read them
 }
 
 // A Poisson draw with mean rho for replica j (Sec. 2, Eq. 1): inversion of
@@ -450,7 +462,9 @@ __device__ __forceinline__ bool round_tie(double rho, double frac, double bounda
     return fabs(__dsub_rn(frac, boundary)) < __dmul_rn(0x1p-48, fmax(1.0, rho));
 }
 
-// One block of 1024 old replicas (chunk): copy numbers and their block scan.
+// One block of old replicas (chunk of blockDim): copy numbers and their block
+// scan.  About 25 FP64 instructions per replica (many more for Poisson draws)
+// at two lanes per clock and SM: small chunks spread them over the SMs.
 // w(E_j) comes from the host table wtab by distance |E_j - E_ref|.
 // j0: global index of local replica 0 (a population shared by several GPUs):
 // the random numbers of replica j follow j0 + j.

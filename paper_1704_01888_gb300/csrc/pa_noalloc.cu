@@ -37,7 +37,8 @@ namespace {
 constexpr int kMaxReplicas = 1 << 18;             // R_prev
 constexpr int kMaxL = 256;                        // lattice size (2N + 1 energy bins)
 constexpr int kMaxBins = 2 * kMaxL * kMaxL + 1;
-constexpr int kMaxBlocks = (kMaxReplicas + 1023) / 1024;
+constexpr int kMaxBlocks = 1024;  // of resample_chunk replicas, whatever the capacity
+static_assert((1 << 17) / 128 <= kMaxBlocks && kMaxReplicas / 256 <= kMaxBlocks, "block sums");
 
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t kOffState = 0;

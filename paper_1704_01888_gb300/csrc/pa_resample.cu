@@ -14,8 +14,6 @@
 //               block-local exclusive scan (warp shuffles).
 //   k_scatter   block offsets, the new population size R_i (checked against
 //               the capacity) and the parent map parent[off_j + c] = j.
-//   k_resample_small  the three stages above in one block, for capacities
-//               of at most 4096 replicas.
 //   k_finalize  Sec. 2 step 4 / Sec. 3 Eq. 4: population averages from exact
 //               integer sums, the fluctuation-formula specific heat, the
 //               magnetisation of Eq. 5, ln Z of Eq. 2 and the family entropy.
@@ -28,6 +26,7 @@ namespace pa {
 namespace {
 
 constexpr int kBlock = 1024;
+constexpr int kWeightsCluster = 8;  // blocks of k_weights (the portable cluster size)
 
 __global__ void k_init(uint32_t *spins, int32_t *anc, int q, int L, int R, uint32_t k0, uint32_t k1,
                        uint32_t stream_hi, int ground, uint32_t slot0)
@@ -38,12 +37,11 @@ __global__ void k_init(uint32_t *spins, int32_t *anc, int q, int L, int R, uint3
         dev::init_item(spins, anc, q, L, i, k0, k1, stream_hi, ground, slot0);
 }
 
-__global__ void __launch_bounds__(kBlock) k_weights(const int32_t *hist, int nbins, double dbeta, const double *wtab,
-                                                    DevState *st, int R_prev_all)
+__global__ void __launch_bounds__(dev::kWeightsThreads) k_weights(const int32_t *hist, int nbins, double dbeta,
+                                                                  const double *wtab, DevState *st, int R_prev_all)
 {
-    __shared__ unsigned long long s_acc[dev::kSumLimbs];
-    __shared__ long long s_l[32];
-    dev::weights_body(hist, nbins, dbeta, wtab, st, s_acc, s_l, R_prev_all);
+    __shared__ dev::WeightsShared sh;
+    dev::weights_body(hist, nbins, dbeta, wtab, st, sh, R_prev_all);
 }
 
 __global__ void __launch_bounds__(kBlock) k_counts(const int32_t *E, int twoN, int R_target, int mode, int step,
@@ -63,38 +61,6 @@ __global__ void __launch_bounds__(kBlock) k_scatter(const int32_t *counts, const
     __shared__ long long s_l[32];
     dev::scatter_body(blockIdx.x, gridDim.x, counts, local_off, blocksum, parent, R_cap, hist_zero, nbins, st, s_l,
                       min_total);
-}
-
-// Small populations (R_cap <= kSmallResample replicas): the three resampling
-// stages in one block, one after the other, with the bodies of k_weights,
-// k_counts and k_scatter run chunk by chunk.  Same arithmetic and the same
-// results; two launches fewer per step where launch latency dominates.
-constexpr int kSmallResample = 4 * kBlock;
-
-__global__ void __launch_bounds__(kBlock) k_resample_small(const int32_t *hist, int nbins, const int32_t *E,
-                                                           double dbeta, int R_target, int R_cap, int mode, int step,
-                                                           uint32_t stream_hi, uint32_t k0, uint32_t k1,
-                                                           const double *wtab, int32_t *counts, int32_t *local_off,
-                                                           int32_t *blocksum, int32_t *parent, int32_t *hist_zero,
-                                                           DevState *st, int j0, int R_prev_all)
-{
-    __shared__ unsigned long long s_acc[dev::kSumLimbs];
-    __shared__ long long s_l[32];
-    __shared__ int s_i[32];
-    dev::weights_body(hist, nbins, dbeta, wtab, st, s_acc, s_l, R_prev_all);
-    __syncthreads();
-    const int nb = (R_cap + kBlock - 1) / kBlock;
-    for (int chunk = 0; chunk < nb; ++chunk) {
-        dev::counts_body(chunk, E, nbins - 1, R_target, mode, step, stream_hi, k0, k1, wtab, counts, local_off,
-                         blocksum, st, s_i, j0);
-        __syncthreads();
-    }
-    const int nb2 = nb > (nbins + kBlock - 1) / kBlock ? nb : (nbins + kBlock - 1) / kBlock;
-    for (int chunk = 0; chunk < nb2; ++chunk) {
-        dev::scatter_body(chunk, nb2, counts, local_off, blocksum, parent, R_cap, hist_zero, nbins, st, s_l,
-                          R_prev_all > 0 ? 0 : 1);
-        __syncthreads();
-    }
 }
 
 __global__ void __launch_bounds__(kBlock) k_finalize(DevState *st, unsigned long long *acc, int32_t *fam, int R0,
@@ -254,19 +220,15 @@ cudaError_t launch_resample(const int32_t *hist, int nbins, const int32_t *E, do
                             int32_t *parent, int32_t *hist_zero, DevState *st, cudaStream_t s, int j0,
                             int R_prev_all)
 {
-    if (R_cap <= kSmallResample) {
-        k_resample_small<<<1, kBlock, 0, s>>>(hist, nbins, E, dbeta, R_target, R_cap, mode, step, stream_hi, k0, k1,
-                                              wtab, counts, local_off, blocksum, parent, hist_zero, st, j0,
-                                              R_prev_all);
-        bump_launch_count(1);
-        return cudaGetLastError();
-    }
-    const int nb = (R_cap + kBlock - 1) / kBlock;
-    k_weights<<<1, kBlock, 0, s>>>(hist, nbins, dbeta, wtab, st, R_prev_all);
-    k_counts<<<nb, kBlock, 0, s>>>(E, nbins - 1, R_target, mode, step, stream_hi, k0, k1, wtab, counts, local_off,
-                                   blocksum, st, j0);
-    const int nb2 = nb > (nbins + kBlock - 1) / kBlock ? nb : (nbins + kBlock - 1) / kBlock;
-    k_scatter<<<nb2, kBlock, 0, s>>>(counts, local_off, blocksum, parent, R_cap, hist_zero, nbins, st,
+    const int threads = resample_chunk(R_cap);
+    const int nb = (R_cap + threads - 1) / threads;
+    const cudaError_t e = launch_clusters(k_weights, kWeightsCluster, kWeightsCluster, dev::kWeightsThreads, 0, s,
+                                          hist, nbins, dbeta, wtab, st, R_prev_all);
+    if (e != cudaSuccess) return e;
+    k_counts<<<nb, threads, 0, s>>>(E, nbins - 1, R_target, mode, step, stream_hi, k0, k1, wtab, counts, local_off,
+                                    blocksum, st, j0);
+    // every block clears its share of the histogram too
+    k_scatter<<<nb, threads, 0, s>>>(counts, local_off, blocksum, parent, R_cap, hist_zero, nbins, st,
                                      R_prev_all > 0 ? 0 : 1);
     bump_launch_count(3);
     return cudaGetLastError();

@@ -17,15 +17,11 @@
 // alpha' = (1/R) sum_{t_j < 1} t_j (<E>_tau - E_j).  The step solves
 // alpha = target by bisection-safeguarded Newton iterations, stopping once
 // |alpha - target| <= 1e-12, and is rounded down to a multiple of 2^-24.
-#include <cooperative_groups.h>
-
 #include <climits>
 #include <mutex>
 
 #include "../../include/pa.h"
-#include "pa_internal.cuh"
-
-namespace cg = cooperative_groups;
+#include "pa_cluster.cuh"
 
 namespace pa {
 
@@ -121,42 +117,6 @@ __device__ __forceinline__ void cluster_sum(cg::cluster_group &cl, double (&v)[N
     for (int i = 0; i < NV; ++i) v[i] = total[i];
 }
 
-// Smallest and largest of lo and hi over the cluster; every thread receives
-// both.  sc: 64 ints, mine: 2 ints read by the other blocks.
-__device__ __forceinline__ void cluster_extremes(cg::cluster_group &cl, int &lo, int &hi, int *sc, int *mine)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    lo = __reduce_min_sync(0xFFFFFFFFu, lo);
-    hi = __reduce_max_sync(0xFFFFFFFFu, hi);
-    if (lane == 0) {
-        sc[warp] = lo;
-        sc[32 + warp] = hi;
-    }
-    __syncthreads();
-    if (warp == 0) {
-        const int l = __reduce_min_sync(0xFFFFFFFFu, lane < nw ? sc[lane] : INT_MAX);
-        const int h = __reduce_max_sync(0xFFFFFFFFu, lane < nw ? sc[32 + lane] : INT_MIN);
-        if (lane == 0) {
-            mine[0] = l;
-            mine[1] = h;
-        }
-    }
-    cl.sync();
-    if (warp == 0) {
-        const int C = (int)cl.num_blocks();
-        const int *theirs = cl.map_shared_rank(mine, lane < C ? lane : 0);
-        const int l = __reduce_min_sync(0xFFFFFFFFu, theirs[0]);
-        const int h = __reduce_max_sync(0xFFFFFFFFu, theirs[1]);
-        if (lane == 0) {
-            sc[0] = l;
-            sc[1] = h;
-        }
-    }
-    __syncthreads();
-    lo = sc[0];
-    hi = sc[1];
-}
-
 // out[0..7] = ln Q, <E>_tau, var_tau(E), <O>_tau, cov_tau(O, E), E_ref, S, k3_tau(E).
 //
 // Bound by FP64: one exp and the moments take about 30 FP64 instructions, 16
@@ -198,7 +158,7 @@ __global__ void __launch_bounds__(kRwThreads) k_rw_forward(const int32_t *__rest
         lo = min(lo, e);
         hi = max(hi, e);
     }
-    cluster_extremes(cl, lo, hi, si, ext);
+    dev::cluster_extremes(cl, lo, hi, si, ext);
     const int ref = lowest ? lo : hi;
     const long long range = (long long)hi - lo + 1;
     double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // S, S1, S2, S3, SO, SOe
@@ -369,7 +329,7 @@ __global__ void __launch_bounds__(kNewtonThreads) k_newton_hist(const int32_t *_
             kmin = min(kmin, k);
             kmax = max(kmax, k);
         }
-    cluster_extremes(cl, kmin, kmax, sh.si, sh.ext);
+    dev::cluster_extremes(cl, kmin, kmax, sh.si, sh.ext);
     const long long range = kmin <= kmax ? (long long)kmax - kmin + 1 : 0;
     const int k0 = kmin + (int)(range * c / C);
     const int m = (int)(range * (c + 1) / C) - (int)(range * c / C);
@@ -480,24 +440,6 @@ struct ClusterSize {
     }
 };
 
-// Launches one cluster of C blocks.
-template <typename... P, typename... A>
-cudaError_t launch_cluster(void (*kernel)(P...), int C, int threads, size_t smem, cudaStream_t s, A... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = C;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
-}
-
 ClusterSize g_rw_cluster, g_newton_cluster;
 
 }  // namespace
@@ -507,7 +449,7 @@ cudaError_t launch_newton(const int32_t *hist, int nbins, const DevState *st, do
 {
     const int C = g_newton_cluster.get(k_newton_hist, kNewtonThreads, 0);
     bump_launch_count(1);
-    return launch_cluster(k_newton_hist, C, kNewtonThreads, 0, s, hist, nbins, st, target, cap, iters, out);
+    return launch_clusters(k_newton_hist, C, C, kNewtonThreads, 0, s, hist, nbins, st, target, cap, iters, out);
 }
 
 }  // namespace pa
@@ -524,7 +466,7 @@ pa_status pa_reweight_forward(const int32_t *E, const double *O, int32_t R, cons
     // a small population does not fill a cluster: one block per 1024 replicas
     int blocks = C;
     while (blocks > 1 && (long long)(blocks / 2) * 1024 >= R) blocks /= 2;
-    return pa::launch_cluster(pa::k_rw_forward, blocks, pa::kRwThreads, smem, (cudaStream_t)stream, E, O, R, dbeta,
+    return pa::launch_clusters(pa::k_rw_forward, blocks, blocks, pa::kRwThreads, smem, (cudaStream_t)stream, E, O, R, dbeta,
                               out) == cudaSuccess
                ? PA_OK
                : PA_ERR_CUDA;
