@@ -113,7 +113,7 @@ struct pa_ctx {
     size_t stage_bytes = 0;
     uint8_t *host_stage = nullptr;  // pinned: device state, one record, the histogram
     double *aux = nullptr;  // small device outputs (Newton step)
-    int32_t *work = nullptr;  // the sweep kernel's group counter
+    int32_t *work = nullptr;  // the sweep kernel's counters (next group, blocks ended)
 
     int step = 0;          // last completed temperature step
     int pending_step = 0;  // step of an enqueued resample awaiting its sweep
@@ -480,7 +480,9 @@ pa::SweepArgs sweep_args(pa_ctx *c, double beta, int theta, int step, int gather
     // few groups per block: hand them out from a counter, so that the blocks
     // end together; with many, equal shares (their ends even out)
     const long long R_est = c->R_fill > 0 ? c->R_fill : c->cfg.R;
-    a.work = R_est < 16LL * c->group * c->grid ? c->work : nullptr;
+    a.dynamic = R_est < 16LL * c->group * c->grid;
+    a.counters = c->work;
+    a.beta = beta;
     return a;
 }
 
@@ -496,11 +498,14 @@ pa_status enqueue_sweep(pa_ctx *c, double beta, int theta, int step)
 {
     const int gather = c->pending_step != 0;
     pa::SweepArgs a = sweep_args(c, beta, theta, step, gather);
+    // family entropies take a block's work over the initial population: a
+    // launch of their own; without them the sweep's last block ends the step
+    if (!c->shard && !a.fam) a.obs = next_obs_slot(c);
     pa_status s = profile_mark(c, 0, true);
     if (s) return s;
     PA_CK(pa::launch_sweep(a, c->threads, c->grid, c->stream));
     if ((s = profile_mark(c, 0, false))) return s;
-    if (!c->shard)
+    if (!c->shard && a.fam)
         PA_CK(pa::launch_finalize(c->st, c->acc, a.fam, c->cfg.R, next_obs_slot(c), beta, c->cfg.q, c->N,
                                   gather, gather, c->stream));
     c->pending_step = 0;
@@ -620,8 +625,10 @@ pa_status ctx_create(const pa_config &g, void *cuda_stream, pa_ctx **out, int ra
         (s = dev_alloc(&c->hist, c->nbins)) || (s = dev_alloc(&c->counts, c->R_cap)) ||
         (s = dev_alloc(&c->local_off, R_child)) || (s = dev_alloc(&c->blocksum, nb)) ||
         (s = dev_alloc(&c->parent, R_child)) || (s = dev_alloc(&c->acc, 4)) || (s = dev_alloc(&c->st, 1)) || (s = dev_alloc(&c->aux, 4)) ||
-        (s = dev_alloc(&c->work, 1)))
+        (s = dev_alloc(&c->work, 2)))
         return fail(s);
+    e = cudaMemsetAsync(c->work, 0, 2 * sizeof(int32_t), c->stream);
+    if (e != cudaSuccess) return fail(cuda_fail(e));
     if (g.track_families) {
         if ((s = dev_alloc(&c->anc[0], c->R_cap)) || (s = dev_alloc(&c->anc[1], c->R_cap)) ||
             (s = dev_alloc(&c->fam, g.R)))

@@ -116,8 +116,10 @@ struct SweepArgs {
     uint32_t stream_hi;        // stream number << 24 (top byte of the slot counter word)
     uint32_t slot0;            // global slot of local slot 0 (0 unless the population spans GPUs)
     int32_t lat;               // 1: the kernel for launches too small to fill the SMs
-    int32_t *work;             // next replica group to hand out (zeroed before each launch), or
-                               // null: each block takes an equal share
+    int32_t dynamic;           // 1: blocks take groups from counters[0]; 0: each block takes an equal share
+    int32_t *counters;         // next replica group, blocks ended; zero before and after each launch
+    DevObs *obs;               // the step's record, written by the last block (null: by launch_finalize)
+    double beta;
 };
 
 // Launchers (pa_sweep.cu)
@@ -191,6 +193,34 @@ void record_cuda_error(const char *msg);
 }  // namespace pa
 
 namespace pa {
+
+// Programmatic dependent launch: the kernels of a temperature step are launched
+// while their predecessor runs (launch_after), so that a launch costs little
+// between them.  A kernel so launched calls wait_prerequisites() before it
+// touches memory; it may let its own successor start at any time, since that
+// waits for it in turn.
+__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_after(void (*kernel)(P...), int cluster, int blocks, int threads, size_t smem, cudaStream_t s,
+                         A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+}
 
 // Philox4x32-10 (Salmon, Moraes, Dror & Shaw, SC'11): ten rounds of two
 // 32x32 -> 64 bit products whose high halves are xored with the other counter

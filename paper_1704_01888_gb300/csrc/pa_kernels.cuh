@@ -347,6 +347,7 @@ __device__ __forceinline__ double exact_round(unsigned long long *acc)
         nonzero |= (unsigned long long)((uint32_t)v != 0u) << i;
     }
     if (!nonzero) return 0.0;
+    if (!nonzero) return 0.0;
     const int t = 63 - __clzll((long long)nonzero);
     int p = 32 * t + 31 - __clz((uint32_t)acc[t]);  // top bit
     const unsigned long long x = limb_bits64(acc, p - 63);  // bit 63 = top bit
@@ -544,20 +545,63 @@ __device__ __forceinline__ void scatter_body(int chunk, int nchunks, const int32
     }
 }
 
-// One block: estimators of the step (Sec. 2 step 4, Eqs. 4-5), family
-// entropy, ln Z of Eq. 2, buffer parity flip.
+// One thread: estimators of the step (Sec. 2 step 4, Eqs. 4-5), ln Z of Eq. 2,
+// buffer parity flip.  S_f, nf: family entropy and count (0 without families).
 // R_all: the population size when the sums and family counts cover several
 // GPUs' replicas (0: this GPU's own).
+__device__ __forceinline__ void finalize_record(DevState *st, unsigned long long *acc, DevObs *obs, double beta, int q,
+                                                int N, int gathered, int resampled, int R_all, double S_f,
+                                                long long nf)
+{
+    const int R_local = gathered ? st->pop_next : st->pop;
+    const int R = R_all > 0 ? R_all : R_local;
+    const long long sE = (long long)acc[0], sE2 = (long long)acc[1], sM = (long long)acc[2];
+    acc[0] = acc[1] = acc[2] = 0ull;
+    const double meanE = (double)sE / (double)R;
+    const double meanE2 = (double)sE2 / (double)R;
+    const double C =
+        __ddiv_rn(__dmul_rn(__dmul_rn(beta, beta), __dsub_rn(meanE2, __dmul_rn(meanE, meanE))), (double)N);
+    const double meanM = (double)((long long)q * sM - (long long)N * R) / __dmul_rn((double)(q - 1), (double)R);
+    double lnQ = 0.0;
+    if (resampled) {
+        lnQ = st->lnQ;
+        st->lnZ = __dadd_rn(st->lnZ, lnQ);
+    }
+    if (gathered) {
+        st->pop = R_local;
+        st->parity ^= 1;
+    }
+    DevObs o;
+    o.beta = beta;
+    o.lnQ = lnQ;
+    o.lnZ = st->lnZ;
+    o.meanE = meanE;
+    o.meanE2 = meanE2;
+    o.C = C;
+    o.meanM = meanM;
+    o.S_f = S_f;
+    o.R = R;
+    o.n_families = nf;
+    // several GPUs: acc[3] holds the near ties summed over them
+    o.n_near_ties = resampled ? (R_all > 0 ? (long long)acc[3] : (long long)st->ties) : 0;
+    if (R_all > 0) acc[3] = 0ull;
+    o.sumE = sE;
+    o.sumE2 = sE2;
+    o.sumMt = sM;
+    *obs = o;
+}
+
+// One block: family entropy, then the estimators.
 __device__ __forceinline__ void finalize_body(DevState *st, unsigned long long *acc, int32_t *fam, int R0, DevObs *obs,
                                               double beta, int q, int N, int gathered, int resampled, double *s_d,
                                               long long *s_l, int R_all = 0)
 {
     if (st->err) return;
-    const int R_local = gathered ? st->pop_next : st->pop;
-    const int R = R_all > 0 ? R_all : R_local;
-    double part = 0.0;
+    const int R = R_all > 0 ? R_all : gathered ? st->pop_next : st->pop;
+    double Sf = 0.0;
     long long nf = 0;
     if (fam) {
+        double part = 0.0;
         for (int f = threadIdx.x; f < R0; f += blockDim.x) {
             const int c = fam[f];
             if (c > 0) {
@@ -567,45 +611,10 @@ __device__ __forceinline__ void finalize_body(DevState *st, unsigned long long *
                 fam[f] = 0;
             }
         }
+        Sf = block_sum_fixed(part, s_d);
+        nf = block_sum_ll(nf, s_l);
     }
-    const double Sf = block_sum_fixed(part, s_d);
-    nf = block_sum_ll(nf, s_l);
-    if (threadIdx.x == 0) {
-        const long long sE = (long long)acc[0], sE2 = (long long)acc[1], sM = (long long)acc[2];
-        acc[0] = acc[1] = acc[2] = 0ull;
-        const double meanE = (double)sE / (double)R;
-        const double meanE2 = (double)sE2 / (double)R;
-        const double C =
-            __ddiv_rn(__dmul_rn(__dmul_rn(beta, beta), __dsub_rn(meanE2, __dmul_rn(meanE, meanE))), (double)N);
-        const double meanM = (double)((long long)q * sM - (long long)N * R) / __dmul_rn((double)(q - 1), (double)R);
-        double lnQ = 0.0;
-        if (resampled) {
-            lnQ = st->lnQ;
-            st->lnZ = __dadd_rn(st->lnZ, lnQ);
-        }
-        if (gathered) {
-            st->pop = R_local;
-            st->parity ^= 1;
-        }
-        DevObs o;
-        o.beta = beta;
-        o.lnQ = lnQ;
-        o.lnZ = st->lnZ;
-        o.meanE = meanE;
-        o.meanE2 = meanE2;
-        o.C = C;
-        o.meanM = meanM;
-        o.S_f = fam ? Sf : 0.0;
-        o.R = R;
-        o.n_families = fam ? nf : 0;
-        // several GPUs: acc[3] holds the near ties summed over them
-        o.n_near_ties = resampled ? (R_all > 0 ? (long long)acc[3] : (long long)st->ties) : 0;
-        if (R_all > 0) acc[3] = 0ull;
-        o.sumE = sE;
-        o.sumE2 = sE2;
-        o.sumMt = sM;
-        *obs = o;
-    }
+    if (threadIdx.x == 0) finalize_record(st, acc, obs, beta, q, N, gathered, resampled, R_all, Sf, nf);
 }
 
 }  // namespace dev

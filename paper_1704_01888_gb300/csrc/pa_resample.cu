@@ -41,6 +41,8 @@ __global__ void __launch_bounds__(dev::kWeightsThreads) k_weights(const int32_t 
                                                                   const double *wtab, DevState *st, int R_prev_all)
 {
     __shared__ dev::WeightsShared sh;
+    launch_dependents();
+    wait_prerequisites();
     dev::weights_body(hist, nbins, dbeta, wtab, st, sh, R_prev_all);
 }
 
@@ -50,6 +52,8 @@ __global__ void __launch_bounds__(kBlock) k_counts(const int32_t *E, int twoN, i
                                                    DevState *st, int j0)
 {
     __shared__ int s_i[32];
+    launch_dependents();
+    wait_prerequisites();
     dev::counts_body(blockIdx.x, E, twoN, R_target, mode, step, stream_hi, k0, k1, wtab, counts, local_off, blocksum,
                      st, s_i, j0);
 }
@@ -59,6 +63,8 @@ __global__ void __launch_bounds__(kBlock) k_scatter(const int32_t *counts, const
                                                     int32_t *hist_zero, int nbins, DevState *st, int min_total)
 {
     __shared__ long long s_l[32];
+    launch_dependents();
+    wait_prerequisites();
     dev::scatter_body(blockIdx.x, gridDim.x, counts, local_off, blocksum, parent, R_cap, hist_zero, nbins, st, s_l,
                       min_total);
 }
@@ -222,16 +228,17 @@ cudaError_t launch_resample(const int32_t *hist, int nbins, const int32_t *E, do
 {
     const int threads = resample_chunk(R_cap);
     const int nb = (R_cap + threads - 1) / threads;
-    const cudaError_t e = launch_clusters(k_weights, kWeightsCluster, kWeightsCluster, dev::kWeightsThreads, 0, s,
-                                          hist, nbins, dbeta, wtab, st, R_prev_all);
-    if (e != cudaSuccess) return e;
-    k_counts<<<nb, threads, 0, s>>>(E, nbins - 1, R_target, mode, step, stream_hi, k0, k1, wtab, counts, local_off,
-                                    blocksum, st, j0);
+    cudaError_t e = launch_after(k_weights, kWeightsCluster, kWeightsCluster, dev::kWeightsThreads, 0, s, hist, nbins,
+                                 dbeta, wtab, st, R_prev_all);
+    if (e == cudaSuccess)
+        e = launch_after(k_counts, 1, nb, threads, 0, s, E, nbins - 1, R_target, mode, step, stream_hi, k0, k1, wtab,
+                         counts, local_off, blocksum, st, j0);
     // every block clears its share of the histogram too
-    k_scatter<<<nb, threads, 0, s>>>(counts, local_off, blocksum, parent, R_cap, hist_zero, nbins, st,
-                                     R_prev_all > 0 ? 0 : 1);
+    if (e == cudaSuccess)
+        e = launch_after(k_scatter, 1, nb, threads, 0, s, counts, local_off, blocksum, parent, R_cap, hist_zero, nbins,
+                         st, R_prev_all > 0 ? 0 : 1);
     bump_launch_count(3);
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_finalize(DevState *st, unsigned long long *acc, int32_t *fam, int R0, DevObs *obs,

@@ -62,13 +62,9 @@ cudaError_t launch_sweep(const SweepArgs &a, int threads, int grid, cudaStream_t
 {
     SweepFn k = pick_kernel(a.q, a.L, a.lat != 0);
     const size_t smem = sweep_smem_bytes(a.q, a.L, a.rpb);
-    if (a.work) {
-        const cudaError_t e = cudaMemsetAsync(a.work, 0, sizeof(int32_t), s);
-        if (e != cudaSuccess) return e;
-    }
-    k<<<grid, threads, smem, s>>>(a);
+    const cudaError_t e = launch_after(k, 1, grid, threads, smem, s, a);
     bump_launch_count(1);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace pa

@@ -4,7 +4,7 @@
 // whole-word rows (pa_sweep.cu) and of the other row geometries
 // (pa_sweep_rows.cu), and the latency kernels (pa_sweep_lat.cu).
 #pragma once
-#include "pa_sweep_body.cuh"
+#include "pa_kernels.cuh"
 
 namespace pa {
 
@@ -68,7 +68,7 @@ __device__ __forceinline__ int2 ticket_range(int t, int R, int rpb, int quantum,
 }
 
 // Persistent blocks over groups of at most rpb replicas of the current
-// population (R_i is known only on the device).  With a.work the blocks take
+// population (R_i is known only on the device).  With a.dynamic the blocks take
 // groups from a counter (for launches of a few groups per block: 1915 against
 // 1845 attempts/ns at q = 10, L = 64, R = 1e5); else each block takes an equal
 // share, counted in quanta of blockDim / (site words per colour) replicas, the
@@ -84,7 +84,9 @@ __device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
     __shared__ uint4 s_tab[dev::kThresholdEntries];
     constexpr int QCAP = LAT ? dev::kLatQueue : B <= 4 ? 384 : dev::kQueueCap;
     __shared__ __align__(16) uint32_t s_queue[dev::queue_words(B, QCAP)];
+    launch_dependents();
     dev::build_threshold_table(s_tab, a.thr);
+    wait_prerequisites();
     DevState *st = a.st;
     if (st->err) return;
     const int parity = st->parity;
@@ -103,8 +105,8 @@ __device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
     for (;;) {
         if (threadIdx.x == 0) {
             int2 g;
-            if (a.work) {
-                g = ticket_range(atomicAdd(a.work, 1), s_R, a.rpb, quantum, gridDim.x);
+            if (a.dynamic) {
+                g = ticket_range(atomicAdd(a.counters, 1), s_R, a.rpb, quantum, gridDim.x);
                 g.y = min(g.y, s_R - g.x);
             } else {
                 g = make_int2(s_next, min(a.rpb, s_end - s_next));
@@ -118,6 +120,16 @@ __device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
         const dev::Group G = make_group(a, parity, g.x, g.y);
         dev::sweep_group_bits<B, MODE, Q, QCAP, LAT>(G, a.L, reinterpret_cast<uint32_t *>(smem4), s_tab, s_queue,
                                                      a.rk0, a.rk1, a.acc);
+    }
+    // the last block to end clears the counters for the next launch and writes
+    // the step's estimators (a launch of its own took 5.5 us and a gap)
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicAdd(a.counters + 1, 1) == (int)gridDim.x - 1) {
+        __threadfence();
+        a.counters[0] = a.counters[1] = 0;
+        if (a.obs && !st->err)
+            dev::finalize_record(st, a.acc, a.obs, a.beta, a.q, a.L * a.L, a.gather, a.gather, 0, 0.0, 0);
     }
 }
 
