@@ -49,7 +49,11 @@ __global__ void k_batch_init(const BatchArgs b)
             if (b.runs[mid].item0 <= i) lo = mid; else hi = mid - 1;
         }
         const RunDev &r = b.runs[lo];
-        dev::init_item(r.buf[0], r.anc[0], r.q, r.L, i - r.item0, b.k0, b.k1, r.stream_hi, r.ground);
+        const long long at = i - r.item0;
+        if (!dev::words_in_order(r.L) || r.ground)
+            dev::init_item(r.buf[0], r.anc[0], r.q, r.L, at, b.k0, b.k1, r.stream_hi, r.ground);
+        else
+            dev::init_words_any(r.buf[0], r.anc[0], r.q, r.L, at, b.k0, b.k1, r.stream_hi);
     }
 }
 
@@ -414,7 +418,7 @@ pa_status pa_batch_create(const pa_run_desc *runs, int32_t M, void *cuda_stream,
         chunk0 += nc;
         b->nchunks[m] = nc;
         r.item0 = item0;
-        item0 += (long long)g.R * (2 * pa::colour_words(g.L));
+        item0 += (long long)g.R * ((pa::dev::words_in_order(g.L) && !r.ground ? 1 : 2) * pa::colour_words(g.L));
         const size_t spin_bytes = (size_t)r.R_cap * pa::replica_bytes(g.q, g.L);
         stage_bytes = std::max(stage_bytes, std::min((size_t)r.R_cap * r.N, (size_t)64 << 20));
         if ((s = balloc(b, &r.buf[0], spin_bytes)) || (s = balloc(b, &r.buf[1], spin_bytes)) ||

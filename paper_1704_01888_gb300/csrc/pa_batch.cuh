@@ -25,7 +25,7 @@ struct RunDev {
     DevObs *obs;  // K + 1 records
     int32_t q, L, N, nbins, R0, R_cap, mode, rpb, chunk0, nchunks, K, ground;
     uint32_t stream_hi;
-    long long item0;  // first site word of this run in the flattened init index
+    long long item0;  // first site word (pair of both colours' words) of this run in the flattened init index
 };
 
 struct StepDev {  // one per (step, run)

@@ -140,12 +140,13 @@ cudaError_t launch_init(uint32_t *spins, int32_t *anc, int q, int L, int R, uint
                         uint32_t stream_hi, int ground, cudaStream_t s, uint32_t slot0 = 0u);
 // wtab: the weight table of dbeta (weight_table below), 2N + 1 entries.
 // j0 / R_prev_all: global index of local replica 0 and the size of the whole
-// population when it spans several GPUs (0, 0 otherwise).
+// population when it spans several GPUs (0, 0 otherwise).  lnQ_out, R_out: where
+// ln Q and the new size (or minus a pa_status) also go (null: nowhere).
 cudaError_t launch_resample(const int32_t *hist, int nbins, const int32_t *E, double dbeta, int R_target,
                             int R_cap, int mode, int step, uint32_t stream_hi, uint32_t k0, uint32_t k1,
                             const double *wtab, int32_t *counts, int32_t *local_off, int32_t *blocksum,
                             int32_t *parent, int32_t *hist_zero, DevState *st, cudaStream_t s, int j0 = 0,
-                            int R_prev_all = 0);
+                            int R_prev_all = 0, double *lnQ_out = nullptr, int32_t *R_out = nullptr);
 // R_all: size of the whole population when the sums cover several GPUs (0 otherwise).
 cudaError_t launch_finalize(DevState *st, unsigned long long *acc, int32_t *fam, int R0, DevObs *obs,
                             double beta, int q, int N, int gathered, int resampled, cudaStream_t s, int R_all = 0);

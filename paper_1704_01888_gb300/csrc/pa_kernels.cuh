@@ -158,6 +158,105 @@ __device__ __forceinline__ void init_item(uint32_t *spins, int32_t *anc, int q, 
     if (rem == 0 && anc) anc[slot] = (int32_t)key_slot;
 }
 
+// Rows of whole words (L a multiple of 64) and packed rows: words w of the two
+// colours together hold the 64 canonical sites 64 w .. 64 w + 63, in order:
+// bit b the sites 64 w + 2 b and 64 w + 2 b + 1, the even one of colour 0 in
+// even rows and of colour 1 in odd rows.
+__host__ __device__ constexpr bool words_in_order(int L) { return L % 64 == 0 || rows_packed(L); }
+
+// Bits of word w whose site lies in an odd row.
+__device__ __forceinline__ uint32_t odd_row_bits(int L, int w)
+{
+    if (L >= 64) return (64 * w / L) & 1 ? 0xFFFFFFFFu : 0u;
+    return L == 32 ? 0xFFFF0000u : L == 16 ? 0xFF00FF00u : 0xF0F0F0F0u;
+}
+
+// Random start of words w of both colours of one replica (words_in_order; i =
+// slot IPC + w): 16 Philox calls of four sites, each made once (init_item makes
+// them for either colour), the states' bits shifted into the planes site by
+// site.  566 -> 149 us for q = 8, L = 128, R = 1e4.
+template <int B>
+__device__ __forceinline__ void init_words(uint32_t *spins, int32_t *anc, int q, int L, long long i, uint32_t k0,
+                                           uint32_t k1, uint32_t stream_hi, uint32_t slot0)
+{
+    constexpr int BP = plane_stride(B);
+    const int IPC = colour_words(L);
+    const int slot = (int)(i / IPC);
+    const int w = (int)(i - (long long)slot * IPC);
+    const uint32_t key_slot = slot0 + (uint32_t)slot;
+    uint32_t even[B], odd[B];
+#pragma unroll
+    for (int p = 0; p < B; ++p) even[p] = odd[p] = 0u;
+#pragma unroll 4
+    for (int c = 0; c < 16; ++c) {
+        const uint4 z = philox10(make_uint4((uint32_t)(16 * w + c), DOM_INIT, 0u, key_slot | stream_hi), k0, k1);
+        uint32_t s[4] = {__umulhi(z.x, (uint32_t)q), __umulhi(z.y, (uint32_t)q), __umulhi(z.z, (uint32_t)q),
+                         __umulhi(z.w, (uint32_t)q)};
+#pragma unroll
+        for (int p = 0; p < B; ++p) {
+            even[p] = __funnelshift_r(even[p], s[0] >> p, 1);
+            even[p] = __funnelshift_r(even[p], s[2] >> p, 1);
+            odd[p] = __funnelshift_r(odd[p], s[1] >> p, 1);
+            odd[p] = __funnelshift_r(odd[p], s[3] >> p, 1);
+        }
+    }
+    const uint32_t m = odd_row_bits(L, w);
+    uint32_t c0[BP], c1[BP];
+#pragma unroll
+    for (int p = 0; p < BP; ++p) {
+        c0[p] = p < B ? (even[p < B ? p : 0] & ~m) | (odd[p < B ? p : 0] & m) : 0u;
+        c1[p] = p < B ? (odd[p < B ? p : 0] & ~m) | (even[p < B ? p : 0] & m) : 0u;
+    }
+    uint32_t *dst = spins + (size_t)slot * replica_words_of(B, L) + (size_t)w * BP;
+    store_planes<BP>(dst, c0);
+    store_planes<BP>(dst + (size_t)IPC * BP, c1);
+    if (w == 0 && anc) anc[slot] = (int32_t)key_slot;
+}
+
+__device__ __forceinline__ void init_words_any(uint32_t *spins, int32_t *anc, int q, int L, long long i, uint32_t k0,
+                                               uint32_t k1, uint32_t stream_hi, uint32_t slot0 = 0u)
+{
+    switch (state_bits(q)) {
+    case 1: init_words<1>(spins, anc, q, L, i, k0, k1, stream_hi, slot0); break;
+    case 2: init_words<2>(spins, anc, q, L, i, k0, k1, stream_hi, slot0); break;
+    case 3: init_words<3>(spins, anc, q, L, i, k0, k1, stream_hi, slot0); break;
+    case 4: init_words<4>(spins, anc, q, L, i, k0, k1, stream_hi, slot0); break;
+    case 5: init_words<5>(spins, anc, q, L, i, k0, k1, stream_hi, slot0); break;
+    case 6: init_words<6>(spins, anc, q, L, i, k0, k1, stream_hi, slot0); break;
+    default: init_words<7>(spins, anc, q, L, i, k0, k1, stream_hi, slot0); break;
+    }
+}
+
+// The 64 canonical sites of words w of both colours (words_in_order; i = slot
+// IPC + w) as bytes: four sites at a time, each plane's bits spread over four
+// bytes by a multiplication.  One site per thread, with divisions, took 136 us
+// for 4000 replicas of 64 x 64 (16 MB); now 11 us.
+__device__ __forceinline__ void canonical_words(const uint32_t *spins, uint8_t *out, int q, int L, long long i)
+{
+    const int B = state_bits(q), BP = plane_stride(B);
+    const int IPC = colour_words(L);
+    const long long r = i / IPC;
+    const int w = (int)(i - r * IPC);
+    const uint32_t *src = spins + (size_t)r * replica_words_of(B, L) + (size_t)w * BP;
+    const uint32_t m = odd_row_bits(L, w);
+    uint32_t v[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = 0u;
+    for (int p = 0; p < B; ++p) {
+        const uint32_t c0 = src[p], c1 = src[(size_t)IPC * BP + p];
+        const uint32_t even = (c0 & ~m) | (c1 & m), odd = (c1 & ~m) | (c0 & m);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            const uint32_t e = (((even >> (2 * j)) & 3u) * 0x8001u) & 0x00010001u;
+            const uint32_t o = (((odd >> (2 * j)) & 3u) * 0x800100u) & 0x01000100u;
+            v[j] |= (e | o) << p;
+        }
+    }
+    uint4 *dst = reinterpret_cast<uint4 *>(out + 64 * i);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) dst[j] = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+}
+
 // One site word (i indexes (slot, colour, word) as in init_item) of the
 // multi-spin-coded layout from a population in the canonical layout
 // [slot][y][x], one byte per spin (the inverse of canonical_state).
@@ -346,7 +445,6 @@ __device__ __forceinline__ double exact_round(unsigned long long *acc)
         carry = v >> 32;
         nonzero |= (unsigned long long)((uint32_t)v != 0u) << i;
     }
-    if (!nonzero) return 0.0;
     if (!nonzero) return 0.0;
     const int t = 63 - __clzll((long long)nonzero);
     int p = 32 * t + 31 - __clz((uint32_t)acc[t]);  // top bit

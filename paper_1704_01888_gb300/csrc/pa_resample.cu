@@ -31,10 +31,15 @@ constexpr int kWeightsCluster = 8;  // blocks of k_weights (the portable cluster
 __global__ void k_init(uint32_t *spins, int32_t *anc, int q, int L, int R, uint32_t k0, uint32_t k1,
                        uint32_t stream_hi, int ground, uint32_t slot0)
 {
-    const long long total = (long long)R * (2 * colour_words(L));
+    const bool pairs = dev::words_in_order(L) && !ground;
+    const long long total = (long long)R * ((pairs ? 1 : 2) * colour_words(L));
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x)
-        dev::init_item(spins, anc, q, L, i, k0, k1, stream_hi, ground, slot0);
+         i += (long long)gridDim.x * blockDim.x) {
+        if (pairs)
+            dev::init_words_any(spins, anc, q, L, i, k0, k1, stream_hi, slot0);
+        else
+            dev::init_item(spins, anc, q, L, i, k0, k1, stream_hi, ground, slot0);
+    }
 }
 
 __global__ void __launch_bounds__(dev::kWeightsThreads) k_weights(const int32_t *hist, int nbins, double dbeta,
@@ -60,13 +65,18 @@ __global__ void __launch_bounds__(kBlock) k_counts(const int32_t *E, int twoN, i
 
 __global__ void __launch_bounds__(kBlock) k_scatter(const int32_t *counts, const int32_t *local_off,
                                                     const int32_t *blocksum, int32_t *parent, int R_cap,
-                                                    int32_t *hist_zero, int nbins, DevState *st, int min_total)
+                                                    int32_t *hist_zero, int nbins, DevState *st, int min_total,
+                                                    double *lnQ_out, int32_t *R_out)
 {
     __shared__ long long s_l[32];
     launch_dependents();
     wait_prerequisites();
     dev::scatter_body(blockIdx.x, gridDim.x, counts, local_off, blocksum, parent, R_cap, hist_zero, nbins, st, s_l,
                       min_total);
+    if (R_out && blockIdx.x == 0 && threadIdx.x == 0) {  // this thread wrote the size or the error
+        *R_out = st->err ? -st->err : st->pop_next;
+        *lnQ_out = st->err ? 0.0 : st->lnQ;
+    }
 }
 
 __global__ void __launch_bounds__(kBlock) k_finalize(DevState *st, unsigned long long *acc, int32_t *fam, int R0,
@@ -187,6 +197,13 @@ __global__ void k_shard_check(DevState *st, int expected)
 
 __global__ void k_to_canonical(const uint32_t *spins, uint8_t *out, int q, int L, long long count)
 {
+    if (dev::words_in_order(L) && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
+        const long long total = count * colour_words(L);
+        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+             i += (long long)gridDim.x * blockDim.x)
+            dev::canonical_words(spins, out, q, L, i);
+        return;
+    }
     const long long total = count * L * L;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x)
@@ -214,7 +231,7 @@ int grid_for(long long work, int threads)
 cudaError_t launch_init(uint32_t *spins, int32_t *anc, int q, int L, int R, uint32_t k0, uint32_t k1,
                         uint32_t stream_hi, int ground, cudaStream_t s, uint32_t slot0)
 {
-    const long long work = (long long)R * (2 * colour_words(L));
+    const long long work = (long long)R * ((dev::words_in_order(L) && !ground ? 1 : 2) * colour_words(L));
     k_init<<<grid_for(work, 256), 256, 0, s>>>(spins, anc, q, L, R, k0, k1, stream_hi, ground, slot0);
     bump_launch_count(1);
     return cudaGetLastError();
@@ -224,7 +241,7 @@ cudaError_t launch_resample(const int32_t *hist, int nbins, const int32_t *E, do
                             int R_cap, int mode, int step, uint32_t stream_hi, uint32_t k0, uint32_t k1,
                             const double *wtab, int32_t *counts, int32_t *local_off, int32_t *blocksum,
                             int32_t *parent, int32_t *hist_zero, DevState *st, cudaStream_t s, int j0,
-                            int R_prev_all)
+                            int R_prev_all, double *lnQ_out, int32_t *R_out)
 {
     const int threads = resample_chunk(R_cap);
     const int nb = (R_cap + threads - 1) / threads;
@@ -236,7 +253,7 @@ cudaError_t launch_resample(const int32_t *hist, int nbins, const int32_t *E, do
     // every block clears its share of the histogram too
     if (e == cudaSuccess)
         e = launch_after(k_scatter, 1, nb, threads, 0, s, counts, local_off, blocksum, parent, R_cap, hist_zero, nbins,
-                         st, R_prev_all > 0 ? 0 : 1);
+                         st, R_prev_all > 0 ? 0 : 1, lnQ_out, R_out);
     bump_launch_count(3);
     return e;
 }
@@ -251,7 +268,7 @@ cudaError_t launch_finalize(DevState *st, unsigned long long *acc, int32_t *fam,
 
 cudaError_t launch_to_canonical(const uint32_t *spins, uint8_t *out, int q, int L, int64_t count, cudaStream_t s)
 {
-    k_to_canonical<<<grid_for(count * L * L, 256), 256, 0, s>>>(spins, out, q, L, count);
+    k_to_canonical<<<grid_for(dev::words_in_order(L) ? count * colour_words(L) : count * L * L, 256), 256, 0, s>>>(spins, out, q, L, count);
     bump_launch_count(1);
     return cudaGetLastError();
 }
@@ -297,7 +314,7 @@ cudaError_t launch_shard_accept(DevState *st, const int32_t *recv_cnt, int n_run
     const int nb = (n_runs + kBlock - 1) / kBlock;
     if (nb > 0) k_shard_run_scan<<<nb, kBlock, 0, s>>>(recv_cnt, n_runs, local_off, blocksum);
     k_scatter<<<nb > 0 ? nb : 1, kBlock, 0, s>>>(recv_cnt, local_off, blocksum, parent, R_cap, hist_zero, nbins, st,
-                                                 0);
+                                                 0, nullptr, nullptr);
     k_shard_check<<<1, 32, 0, s>>>(st, n_expected);
     bump_launch_count(nb > 0 ? 4 : 3);
     return cudaGetLastError();
