@@ -11,6 +11,7 @@
 // of a batch reproduces bit for bit a lone run (pa_init) with the same
 // configuration; block shapes chosen by the autotuner never change results.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -19,6 +20,8 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/pa.h"
@@ -127,6 +130,11 @@ struct pa_batch {
     int32_t *counter_d = nullptr;
     int32_t *work_d = nullptr;   // 2 x (Kmax + 1) group counters of the sweep kernel's two parts
     int32_t *order_d = nullptr;  // run order of the sweep kernel's groups
+    pa::DevState *st_all = nullptr;  // the runs' states, histograms and sums, each in one array
+    std::vector<pa::DevState> st_start;
+    int32_t *hist_all = nullptr;
+    unsigned long long *acc_all = nullptr;
+    size_t bins_total = 0;
     std::vector<void *> allocs;
     pa::BatchArgs args{};
     int smem_budget = 65536, threads = 512, grid = 0, sms = 0;
@@ -237,18 +245,11 @@ pa_status enqueue_start(pa_batch *b)
 {
     PB_CK(cudaMemsetAsync(b->counter_d, 0, sizeof(int32_t), b->stream));
     PB_CK(cudaMemsetAsync(b->work_d, 0, sizeof(int32_t) * 2 * (size_t)(b->Kmax + 1), b->stream));
-    for (int m = 0; m < b->M; ++m) {
-        const pa::RunDev &r = b->runs_h[m];
-        pa::DevState h{};
-        h.pop = b->cfg[m].R;
-        h.lnZ = b->cfg[m].init_mode == PA_INIT_GROUND ? std::log((double)r.q) - b->cfg[m].beta0 * (double)(-2 * r.N)
-                                                       : (double)r.N * std::log((double)r.q);
-        PB_CK(cudaMemcpyAsync(r.st, &h, sizeof(h), cudaMemcpyHostToDevice, b->stream));
-        PB_CK(cudaMemsetAsync(r.hist, 0, sizeof(int32_t) * r.nbins, b->stream));
-        PB_CK(cudaMemsetAsync(r.acc, 0, sizeof(unsigned long long) * 3, b->stream));
+    PB_CK(cudaMemcpyAsync(b->st_all, b->st_start.data(), sizeof(pa::DevState) * b->M, cudaMemcpyHostToDevice, b->stream));
+    PB_CK(cudaMemsetAsync(b->hist_all, 0, sizeof(int32_t) * b->bins_total, b->stream));
+    PB_CK(cudaMemsetAsync(b->acc_all, 0, sizeof(unsigned long long) * 3 * b->M, b->stream));
+    for (const pa::RunDev &r : b->runs_h)
         if (r.fam) PB_CK(cudaMemsetAsync(r.fam, 0, sizeof(int32_t) * r.R0, b->stream));
-        PB_CK(cudaStreamSynchronize(b->stream));  // h lives on this stack frame
-    }
     long long threads_total = (b->args.total_items + 255) / 256;
     int grid = (int)std::min<long long>(threads_total, 65535LL * 16);
     pa::k_batch_init<<<grid, 256, 0, b->stream>>>(b->args);
@@ -279,11 +280,10 @@ pa_status enqueue_step(pa_batch *b, cudaStream_t s)
 
 pa_status check_runs(const pa_batch *b)
 {
-    for (int m = 0; m < b->M; ++m) {
-        pa::DevState h;
-        PB_CK(cudaMemcpy(&h, b->runs_h[m].st, sizeof(h), cudaMemcpyDeviceToHost));
-        if (h.err) return (pa_status)h.err;
-    }
+    std::vector<pa::DevState> h(b->M);
+    PB_CK(cudaMemcpy(h.data(), b->st_all, sizeof(pa::DevState) * b->M, cudaMemcpyDeviceToHost));
+    for (const pa::DevState &s : h)
+        if (s.err) return (pa_status)s.err;
     return PA_OK;
 }
 
@@ -338,6 +338,29 @@ void cache_file_store(const std::string &key, int budget, int threads)
     if (!f) return;
     std::fprintf(f, "%s\t%d\t%d\n", key.c_str(), budget, threads);
     std::fclose(f);
+}
+
+// Computes the weight tables on up to eight threads (fewer where the system
+// refuses one), each taking the next table from a counter.
+template <typename Table>
+void fill_tables(const std::vector<Table> &tables)
+{
+    size_t entries = 0;
+    for (const Table &t : tables) entries += (size_t)t.n;
+    std::atomic<size_t> next{0};
+    auto work = [&]() {
+        for (size_t i; (i = next.fetch_add(1)) < tables.size();)
+            pa::weight_table(tables[i].dbeta, tables[i].n, tables[i].out);
+    };
+    const unsigned want = (unsigned)std::min<size_t>(8, entries / 32768);
+    std::vector<std::thread> threads;
+    try {
+        threads.reserve(8);
+        for (unsigned k = 1; k < std::min(want, std::thread::hardware_concurrency()); ++k) threads.emplace_back(work);
+    } catch (...) {  // no thread to be had: those that run and this one do the work
+    }
+    work();
+    for (std::thread &t : threads) t.join();
 }
 
 }  // namespace
@@ -419,20 +442,56 @@ pa_status pa_batch_create(const pa_run_desc *runs, int32_t M, void *cuda_stream,
         b->nchunks[m] = nc;
         r.item0 = item0;
         item0 += (long long)g.R * ((pa::dev::words_in_order(g.L) && !r.ground ? 1 : 2) * pa::colour_words(g.L));
-        const size_t spin_bytes = (size_t)r.R_cap * pa::replica_bytes(g.q, g.L);
         stage_bytes = std::max(stage_bytes, std::min((size_t)r.R_cap * r.N, (size_t)64 << 20));
-        if ((s = balloc(b, &r.buf[0], spin_bytes)) || (s = balloc(b, &r.buf[1], spin_bytes)) ||
-            (s = balloc(b, &r.E, r.R_cap)) || (s = balloc(b, &r.Mt, r.R_cap)) || (s = balloc(b, &r.hist, r.nbins)) ||
-            (s = balloc(b, &r.counts, r.R_cap)) || (s = balloc(b, &r.local_off, r.R_cap)) ||
-            (s = balloc(b, &r.blocksum, nc)) || (s = balloc(b, &r.parent, r.R_cap)) ||
-            (s = balloc(b, &r.acc, 3)) || (s = balloc(b, &r.st, 1)) ||
-            (s = balloc(b, &r.obs, (size_t)d.K + 1)))
-            return fail(s);
-        if (g.track_families) {
-            if ((s = balloc(b, &r.anc[0], r.R_cap)) || (s = balloc(b, &r.anc[1], r.R_cap)) ||
-                (s = balloc(b, &r.fam, g.R)))
-                return fail(s);
+        b->bins_total += (size_t)r.nbins;
+    }
+    // the runs' arrays from one allocation (a call per array and run held the
+    // creation up for milliseconds), laid out twice: for their sizes, then in place
+    size_t arena_bytes = 0;
+    unsigned char *arena = nullptr;
+    auto take = [&](auto **p, size_t count) {
+        using T = std::remove_reference_t<decltype(**p)>;
+        *p = arena ? reinterpret_cast<T *>(arena + arena_bytes) : nullptr;
+        arena_bytes += (std::max<size_t>(count, 1) * sizeof(T) + 255) / 256 * 256;
+    };
+    auto lay_out = [&]() {
+        arena_bytes = 0;
+        for (int m = 0; m < M; ++m) {
+            pa::RunDev &r = b->runs_h[m];
+            const size_t spin_words = (size_t)r.R_cap * pa::replica_words(r.q, r.L);
+            take(&r.buf[0], spin_words);
+            take(&r.buf[1], spin_words);
+            take(&r.E, r.R_cap);
+            take(&r.Mt, r.R_cap);
+            take(&r.counts, r.R_cap);
+            take(&r.local_off, r.R_cap);
+            take(&r.blocksum, b->nchunks[m]);
+            take(&r.parent, r.R_cap);
+            take(&r.obs, (size_t)r.K + 1);
+            if (b->cfg[m].track_families) {
+                take(&r.anc[0], r.R_cap);
+                take(&r.anc[1], r.R_cap);
+                take(&r.fam, r.R0);
+            }
         }
+        take(&b->st_all, M);
+        take(&b->hist_all, b->bins_total);
+        take(&b->acc_all, 3 * (size_t)M);
+    };
+    lay_out();
+    if ((s = balloc(b, &arena, arena_bytes))) return fail(s);
+    lay_out();
+    b->st_start.assign(M, pa::DevState{});
+    size_t bin0 = 0;
+    for (int m = 0; m < M; ++m) {
+        pa::RunDev &r = b->runs_h[m];
+        r.st = b->st_all + m;
+        r.hist = b->hist_all + bin0;
+        r.acc = b->acc_all + 3 * (size_t)m;
+        bin0 += (size_t)r.nbins;
+        b->st_start[m].pop = r.R0;
+        b->st_start[m].lnZ = r.ground ? std::log((double)r.q) - b->cfg[m].beta0 * (double)(-2 * r.N)
+                                      : (double)r.N * std::log((double)r.q);
     }
     b->n_parts = (int)b->has_part[0] + (int)b->has_part[1];
     // weight tables: one per run and distinct dbeta of its schedule (a
@@ -447,14 +506,22 @@ pa_status pa_batch_create(const pa_run_desc *runs, int32_t M, void *cuda_stream,
             if (wt_at[m].emplace(key, wt_total).second) wt_total += (size_t)b->runs_h[m].nbins;
         }
     }
+    // a table is thousands of exps of the C library: a few threads share the tables
     std::vector<double> wt_host(wt_total);
+    struct Table {
+        double dbeta;
+        int n;
+        double *out;
+    };
+    std::vector<Table> tables;
     for (int m = 0; m < M; ++m) {
         for (const auto &kv : wt_at[m]) {
             double dbeta;
             std::memcpy(&dbeta, &kv.first, sizeof(dbeta));
-            pa::weight_table(dbeta, b->runs_h[m].nbins, wt_host.data() + kv.second);
+            tables.push_back({dbeta, b->runs_h[m].nbins, wt_host.data() + kv.second});
         }
     }
+    fill_tables(tables);
     double *wt_dev = nullptr;
     if ((s = balloc(b, &wt_dev, wt_total))) return fail(s);
     e = cudaMemcpy(wt_dev, wt_host.data(), sizeof(double) * wt_total, cudaMemcpyHostToDevice);

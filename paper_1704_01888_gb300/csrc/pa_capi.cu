@@ -99,6 +99,7 @@ struct pa_ctx {
     std::vector<cudaEvent_t> wt_stage_done;     // upload from each staging slot done
     std::vector<uint64_t> wt_key;               // dbeta bits held by each arena slot
     std::vector<long long> wt_stamp;            // last use (0: empty)
+    std::vector<int> wt_len;                    // entries held by each arena slot (nbins, or fewer)
     long long wt_clock = 0;
     int wt_next_stage = 0;
     double *wt_run = nullptr;                   // tables of a long pa_run schedule
@@ -113,6 +114,9 @@ struct pa_ctx {
     size_t stage_bytes = 0;
     uint8_t *host_stage = nullptr;  // pinned: device state, one record, the histogram
     double *aux = nullptr;  // small device outputs (Newton step)
+    int hist_span = 0;      // bins from the lowest to the highest occupied one at the last pa_next_dbeta
+    int32_t *hstore = nullptr;  // histograms taken by pa_run
+    size_t hstore_cap = 0;
     int32_t *work = nullptr;  // the sweep kernel's counters (next group, blocks ended)
 
     int step = 0;          // last completed temperature step
@@ -209,6 +213,7 @@ pa_status alloc_wtables(pa_ctx *c)
         if ((e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) return cuda_fail(e);
     c->wt_key.assign(kWTableSlots, 0);
     c->wt_stamp.assign(kWTableSlots, 0);
+    c->wt_len.assign(kWTableSlots, 0);
     return PA_OK;
 }
 
@@ -234,9 +239,11 @@ void release_run_tables(pa_ctx *c)
 
 // The device weight table of dbeta: a schedule's own tables during a long
 // pa_run, else the arena slot holding it, else a new table in the least
-// recently used slot.
-pa_status get_wtable(pa_ctx *c, double dbeta, const double **out)
+// recently used slot.  need: entries that the step can look up, all of them or
+// the span of the occupied bins where the host knows it (0: all).
+pa_status get_wtable(pa_ctx *c, double dbeta, const double **out, int need = 0)
 {
+    if (need <= 0 || need > c->nbins) need = c->nbins;
     uint64_t key;
     std::memcpy(&key, &dbeta, sizeof(key));
     for (const auto &kv : c->wt_run_at) {
@@ -249,9 +256,13 @@ pa_status get_wtable(pa_ctx *c, double dbeta, const double **out)
     int slot = 0;
     for (int i = 0; i < kWTableSlots; ++i) {
         if (c->wt_stamp[i] && c->wt_key[i] == key) {
-            c->wt_stamp[i] = ++c->wt_clock;
-            *out = c->wt_arena + n * i;
-            return PA_OK;
+            if (c->wt_len[i] >= need) {
+                c->wt_stamp[i] = ++c->wt_clock;
+                *out = c->wt_arena + n * i;
+                return PA_OK;
+            }
+            slot = i;  // too short for this step: computed again in its place
+            break;
         }
         if (c->wt_stamp[i] < c->wt_stamp[slot]) slot = i;
     }
@@ -259,11 +270,13 @@ pa_status get_wtable(pa_ctx *c, double dbeta, const double **out)
     c->wt_next_stage = (k + 1) % kWStage;
     double *host = c->wt_stage + n * k;
     PA_CK(cudaEventSynchronize(c->wt_stage_done[k]));  // its previous upload has left
-    pa::weight_table(dbeta, c->nbins, host);
+    pa::weight_table(dbeta, need, host);
     double *dev = c->wt_arena + n * slot;
-    PA_CK(cudaMemcpyAsync(dev, host, sizeof(double) * n, cudaMemcpyHostToDevice, c->stream));
+    c->wt_stamp[slot] = 0;  // no table until the copy is enqueued
+    PA_CK(cudaMemcpyAsync(dev, host, sizeof(double) * need, cudaMemcpyHostToDevice, c->stream));
     PA_CK(cudaEventRecord(c->wt_stage_done[k], c->stream));
     c->wt_key[slot] = key;
+    c->wt_len[slot] = need;
     c->wt_stamp[slot] = ++c->wt_clock;
     *out = dev;
     return PA_OK;
@@ -282,7 +295,7 @@ void release(pa_ctx *c)
     if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
     void *ptrs[] = {c->spins[0], c->spins[1], c->anc[0], c->anc[1], c->E, c->Mt, c->hist, c->fam,
                     c->counts, c->local_off, c->blocksum, c->parent, c->acc, c->st, c->obs,
-                    c->stage, c->aux, c->work};
+                    c->stage, c->aux, c->hstore, c->work};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (c->host_stage) cudaFreeHost(c->host_stage);
@@ -514,10 +527,10 @@ pa_status enqueue_sweep(pa_ctx *c, double beta, int theta, int step)
     return PA_OK;
 }
 
-pa_status enqueue_resample(pa_ctx *c, double dbeta, int step)
+pa_status enqueue_resample(pa_ctx *c, double dbeta, int step, int table = 0)
 {
     const double *wtab = nullptr;
-    pa_status s = get_wtable(c, dbeta, &wtab);
+    pa_status s = get_wtable(c, dbeta, &wtab, table);
     if (s) return s;
     if ((s = profile_mark(c, 1, true))) return s;
     PA_CK(pa::launch_resample(c->hist, c->nbins, c->E, dbeta, c->cfg.R, c->R_cap, c->cfg.resample_mode, step,
@@ -540,6 +553,21 @@ pa_status sync_state(pa_ctx *c, pa::DevState *out)
         c->failed = true;
         return (pa_status)h.err;
     }
+    return PA_OK;
+}
+
+// Copies the estimator records first .. first + count - 1 (of all written so
+// far) to the host: at most two copies, the ring's two ends, and one wait.
+pa_status copy_records(pa_ctx *c, long long first, int32_t count, pa_obs *out)
+{
+    static_assert(sizeof(pa::DevObs) == sizeof(pa_obs), "pa_obs layout");
+    for (int32_t i = 0; i < count;) {
+        const int at = (int)((first + i) % c->obs_cap);
+        const int run = std::min(c->obs_cap - at, (int)(count - i));
+        PA_CK(cudaMemcpyAsync(out + i, c->obs + at, sizeof(pa_obs) * run, cudaMemcpyDeviceToHost, c->stream));
+        i += run;
+    }
+    PA_CK(cudaStreamSynchronize(c->stream));
     return PA_OK;
 }
 
@@ -615,12 +643,12 @@ pa_status ctx_create(const pa_config &g, void *cuda_stream, pa_ctx **out, int ra
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return fail(cuda_fail(e));
 
-    const size_t spin_bytes = (size_t)c->R_cap * pa::replica_bytes(g.q, g.L);
+    const size_t spin_words = (size_t)c->R_cap * pa::replica_words(g.q, g.L);
     // a shard's children (parent map, run scan) can number up to the whole
     // population's capacity, its own replicas only up to its share
     const int R_child = (int)R_cap;
     const int nb = std::max((R_child + 1023) / 1024, pa::resample_blocks(R_child));
-    if ((s = dev_alloc(&c->spins[0], spin_bytes)) || (s = dev_alloc(&c->spins[1], spin_bytes)) ||
+    if ((s = dev_alloc(&c->spins[0], spin_words)) || (s = dev_alloc(&c->spins[1], spin_words)) ||
         (s = dev_alloc(&c->E, c->R_cap)) || (s = dev_alloc(&c->Mt, c->R_cap)) ||
         (s = dev_alloc(&c->hist, c->nbins)) || (s = dev_alloc(&c->counts, c->R_cap)) ||
         (s = dev_alloc(&c->local_off, R_child)) || (s = dev_alloc(&c->blocksum, nb)) ||
@@ -960,16 +988,7 @@ pa_status pa_observables_history(pa_ctx *c, int32_t count, pa_obs *out)
     if (count > c->n_obs || count > c->obs_cap) return PA_ERR_INVALID;
     pa_status s = sync_state(c, nullptr);
     if (s) return s;
-    for (int32_t i = 0; i < count;) {
-        const long long rec = c->n_obs - count + i;
-        const int at = (int)(rec % c->obs_cap);
-        int run = c->obs_cap - at;
-        if (run > count - i) run = count - i;
-        PA_CK(cudaMemcpyAsync(out + i, c->obs + at, sizeof(pa_obs) * run, cudaMemcpyDeviceToHost, c->stream));
-        i += run;
-    }
-    PA_CK(cudaStreamSynchronize(c->stream));
-    return PA_OK;
+    return copy_records(c, c->n_obs - count, count, out);
 }
 
 pa_status pa_population_size(pa_ctx *c, int32_t *R_out)
@@ -1295,11 +1314,15 @@ pa_status pa_run(pa_ctx *c, const double *betas, int32_t K, int32_t theta, pa_ob
         c->obs_cap = K + 1;
         c->n_obs = 1;
     }
-    int32_t *hstore = nullptr;
-    if (n_hist > 0) {
-        pa_status s = dev_alloc(&hstore, (size_t)n_hist * c->nbins);
+    if (n_hist > 0 && (size_t)n_hist * c->nbins > c->hstore_cap) {
+        PA_CK(cudaStreamSynchronize(c->stream));
+        if (c->hstore) cudaFree(c->hstore);
+        c->hstore_cap = 0;
+        pa_status s = dev_alloc(&c->hstore, (size_t)n_hist * c->nbins);
         if (s) return s;
+        c->hstore_cap = (size_t)n_hist * c->nbins;
     }
+    int32_t *const hstore = c->hstore;
     const long long first_obs = c->n_obs;
     const int step0 = c->step;
     // every weight table of the schedule is on the device before any capture
@@ -1340,7 +1363,6 @@ pa_status pa_run(pa_ctx *c, const double *betas, int32_t K, int32_t theta, pa_ob
         }
         if (s) {
             release_run_tables(c);
-            if (hstore) cudaFree(hstore);
             return s;
         }
     }
@@ -1360,7 +1382,6 @@ pa_status pa_run(pa_ctx *c, const double *betas, int32_t K, int32_t theta, pa_ob
         if (e != cudaSuccess) {
             c->profiling = was_profiling;
             release_run_tables(c);
-            if (hstore) cudaFree(hstore);
             return cuda_fail(e);
         }
         c->stream = c->capture_stream;
@@ -1389,22 +1410,12 @@ pa_status pa_run(pa_ctx *c, const double *betas, int32_t K, int32_t theta, pa_ob
     if (graph) cudaGraphDestroy(graph);
     cudaStreamSynchronize(c->stream);
     release_run_tables(c);
-    if (s == PA_OK && obs_out) {
-        for (int i = 0; i < K; ++i) {
-            const pa::DevObs *slot = c->obs + ((first_obs + i) % c->obs_cap);
-            cudaError_t e = cudaMemcpy(obs_out + i, slot, sizeof(pa_obs), cudaMemcpyDeviceToHost);
-            if (e != cudaSuccess) {
-                s = cuda_fail(e);
-                break;
-            }
-        }
-    }
+    if (s == PA_OK && obs_out) s = copy_records(c, first_obs, K, obs_out);
     if (s == PA_OK && n_hist > 0) {
         cudaError_t e = cudaMemcpy(hist_out, hstore, sizeof(int32_t) * (size_t)n_hist * c->nbins,
                                    cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) s = cuda_fail(e);
     }
-    if (hstore) cudaFree(hstore);
     return s;
 }
 
@@ -1417,11 +1428,12 @@ pa_status pa_next_dbeta(pa_ctx *c, double target, double dbeta_cap, int32_t iter
     if (c->shard) return PA_ERR_STATE;
     if (c->failed || c->pending_step != 0) return PA_ERR_STATE;
     PA_CK(pa::launch_newton(c->hist, c->nbins, c->st, target, dbeta_cap, iters, c->aux, c->stream));
-    double h[2];
+    double h[3];
     PA_CK(cudaMemcpyAsync(h, c->aux, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
     pa_status s = sync_state(c, nullptr);
     if (s) return s;
     *dbeta_out = h[0];
+    c->hist_span = (int)h[2];
     return PA_OK;
 }
 
@@ -1455,19 +1467,16 @@ pa_status pa_run_adaptive(pa_ctx *c, double beta_end, double target, double dbet
         if (s) return s;
         const double nb = (dbeta == room) ? beta_end : beta + dbeta;
         const int step = c->step + 1;
-        if ((s = enqueue_resample(c, dbeta, step)) || (s = enqueue_sweep(c, nb, theta, step))) return s;
+        // the step's weights reach as far as its occupied bins: at L = 128 some
+        // 2000 of the 32769 exps that held the GPU up for 160 us per step
+        if ((s = enqueue_resample(c, dbeta, step, c->hist_span)) || (s = enqueue_sweep(c, nb, theta, step))) return s;
         K += 1;
         if (betas_out) betas_out[K - 1] = nb;
         beta = nb;
     }
     pa_status s = sync_state(c, nullptr);
     if (s) return s;
-    if (obs_out) {
-        for (int i = 0; i < K; ++i) {
-            const pa::DevObs *slot = c->obs + ((first_obs + i) % c->obs_cap);
-            PA_CK(cudaMemcpy(obs_out + i, slot, sizeof(pa_obs), cudaMemcpyDeviceToHost));
-        }
-    }
+    if (obs_out && (s = copy_records(c, first_obs, K, obs_out))) return s;
     *K_out = K;
     return PA_OK;
 }

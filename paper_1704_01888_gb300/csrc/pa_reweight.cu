@@ -395,6 +395,7 @@ __global__ void __launch_bounds__(kNewtonThreads) k_newton_hist(const int32_t *_
     if (c == 0 && tid == 0) {
         out[0] = x;
         out[1] = a;
+        out[2] = (double)range;  // bins from the lowest to the highest occupied one
     }
     cl.sync();  // the blocks' shared memory stays until every reader is done
 }
