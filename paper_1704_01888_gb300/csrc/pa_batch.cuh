@@ -159,9 +159,9 @@ __global__ void __launch_bounds__(1024) k_batch_sweep(const BatchArgs b)
         G.stream_hi = r.stream_hi;
         G.gather = b.gather != 0;
         G.write_back = b.gather || sp.theta > 0;
+        G.err = &r.st->err;
 #if PA_CHECKED
         G.src_limit = r.st->pop;
-        G.err = &r.st->err;
 #endif
         dev::build_threshold_table(s_tab, sp.thr);
         uint32_t *sw = reinterpret_cast<uint32_t *>(smem4);
@@ -177,6 +177,7 @@ __global__ void __launch_bounds__(1024) k_batch_sweep(const BatchArgs b)
         else
             batch_body<2, PART>(r.q, B, G, r.L, sw, s_tab, s_queue, b, r.acc);
     }
+    if (threadIdx.x == 0) dev::bulk_stores_done();
 }
 
 }  // namespace

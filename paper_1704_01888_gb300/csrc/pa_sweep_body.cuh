@@ -271,11 +271,69 @@ struct Group {
     int q, theta, step;
     uint32_t stream_hi;      // stream number << 24, or'ed into the slot counter word
     bool gather, write_back;
+    int32_t *err;            // the run's error flag
 #if PA_CHECKED
     int src_limit;           // a gather's parent slots lie in [0, src_limit)
-    int32_t *err;            // the run's error flag
 #endif
 };
+
+// ---- Bulk copies of whole replicas (cp.async.bulk: 16-byte aligned, sizes
+// multiples of 16 bytes, as replicas are) -----------------------------------
+__device__ __forceinline__ uint32_t shared_address(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+// Orders this thread's accesses to shared memory before bulk copies that touch
+// the same bytes after the next barrier.
+__device__ __forceinline__ void fence_bulk() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+__device__ __forceinline__ void bulk_barrier_init(uint32_t bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(__cvta_generic_to_global(src)), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+
+// Waits for the barrier's bytes, at most about a second (kBulkClocks); false if
+// they did not come.
+constexpr long long kBulkClocks = 2000000000ll;
+__device__ __forceinline__ bool bulk_wait(uint32_t bar)
+{
+    const long long start = clock64();
+    for (;;) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(done)
+            : "r"(bar)
+            : "memory");
+        if (done) return true;
+        if (clock64() - start > kBulkClocks) return false;
+    }
+}
+
+__device__ __forceinline__ void bulk_store(void *dst, uint32_t src, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(__cvta_generic_to_global(dst)),
+                 "r"(src), "r"(bytes)
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
+// The issuing thread: until its bulk stores have read shared memory / are done.
+__device__ __forceinline__ void bulk_stores_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_stores_done() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+
+// Smallest replica that a gather copies in bulk, one copy each; smaller ones
+// are gathered by the threads.
+constexpr uint32_t kBulkReplica = 512;
 
 __device__ __forceinline__ void record_replica(const Group &G, int slot, int E, int Mt, int N, long long &sE,
                                                long long &sE2, long long &sM)
@@ -547,23 +605,59 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
     const int first = G.first, nrep = G.nrep;
     uint4 *smem4 = reinterpret_cast<uint4 *>(sw);
 
-    // gather: replica first + r comes from its parent's lattice
-    for (int i = tid; i < nrep * UPR; i += blockDim.x) {
-        const int r = i / UPR;
-        const int o = i - r * UPR;
+    // Load: replica first + r comes from its parent's lattice.  All copies of
+    // the group are in flight at once; a loop of dependent loads (parent, then
+    // lattice) per 16 bytes took about 15 us per group of 48 lattices of 2 KB.
+    __shared__ __align__(8) unsigned long long s_bar;
+    const uint32_t bar = shared_address(&s_bar), RB = (uint32_t)RW * 4u;
+    auto source = [&](int r) {
         const int slot = first + r;
-#if PA_CHECKED
         int src = G.gather ? G.parent[slot] : slot;
+#if PA_CHECKED
         if (G.gather && (src < 0 || src >= G.src_limit)) {
             atomicExch(G.err, 1);  // PA_ERR_INVALID
             src = 0;
         }
-#else
-        const int src = G.gather ? G.parent[slot] : slot;
 #endif
-        smem4[r * UPR + o] = reinterpret_cast<const uint4 *>(G.in + (size_t)src * RW)[o];
+        return G.in + (size_t)src * RW;
+    };
+    // (the latency kernel's few pieces per thread are quicker by hand)
+    const bool bulk = !LAT && (!G.gather || RB >= kBulkReplica);
+    if (bulk) {
+        if (tid == 0) bulk_barrier_init(bar, RB * (uint32_t)nrep);
+        __syncthreads();
+        if (!G.gather) {
+            if (tid == 0) bulk_load(shared_address(sw), source(0), RB * (uint32_t)nrep, bar);
+        } else {
+            for (int r = tid; r < nrep; r += blockDim.x) bulk_load(shared_address(sw + r * RW), source(r), RB, bar);
+        }
+        const bool ok = bulk_wait(bar);
+        if (__syncthreads_or(!ok)) {
+            // not expected to happen: report it, give the copies once more the
+            // time to land, and leave the group
+            if (tid == 0) atomicExch(G.err, 4);  // PA_ERR_TIMEOUT
+            bulk_wait(bar);
+            __syncthreads();
+            return;
+        }
+        if (tid == 0) asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+    } else {
+        constexpr int U4 = 4;  // 16-byte pieces in flight per thread
+        const uint32_t inv_upr = div_inverse(UPR);
+        const int pieces = nrep * UPR, step = (int)blockDim.x;
+        for (int i0 = tid; i0 < pieces; i0 += U4 * step) {
+            uint4 v[U4];
+#pragma unroll
+            for (int u = 0; u < U4; ++u) {
+                const int i = min(i0 + u * step, pieces - 1), r = div_by(i, inv_upr);
+                v[u] = reinterpret_cast<const uint4 *>(source(r))[i - r * UPR];
+            }
+#pragma unroll
+            for (int u = 0; u < U4; ++u)
+                if (i0 + u * step < pieces) smem4[i0 + u * step] = v[u];
+        }
+        __syncthreads();
     }
-    __syncthreads();
 
     // q and q - 1 as plane masks, for the proposal
     uint32_t qm[B + 1], q1m[B + 1];
@@ -744,6 +838,17 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
         }
     }
 
+    // Write back: the group's replicas lie one after the other on both sides, one
+    // bulk copy that runs beside the measurements (which only read)
+    if (G.write_back && LAT) {
+        uint4 *out4 = reinterpret_cast<uint4 *>(G.out + (size_t)first * RW);
+        for (int i = tid; i < nrep * UPR; i += blockDim.x) out4[i] = smem4[i];
+    } else if (G.write_back) {
+        fence_bulk();
+        __syncthreads();
+        if (tid == 0) bulk_store(G.out + (size_t)first * RW, shared_address(sw), RB * (uint32_t)nrep);
+    }
+
     // sums of the replicas this warp records (lane 0), added up per group: kept
     // over the groups they would take six registers through the sweeps
     long long sE = 0, sE2 = 0, sM = 0;
@@ -827,13 +932,9 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
     }
     if (lane == 0 && (sE | sE2 | sM)) accumulate_totals(totals, sE, sE2, sM);
     group_families(G);
-    __syncthreads();
-    if (G.write_back) {
-        for (int i = tid; i < nrep * UPR; i += blockDim.x) {
-            const int r = i / UPR;
-            const int o = i - r * UPR;
-            reinterpret_cast<uint4 *>(G.out + (size_t)(first + r) * RW)[o] = smem4[r * UPR + o];
-        }
+    if constexpr (!LAT) {
+        fence_bulk();  // the next group's copies overwrite what was read here
+        if (tid == 0) bulk_stores_read();
     }
     __syncthreads();
 }

@@ -45,9 +45,9 @@ __device__ __forceinline__ dev::Group make_group(const SweepArgs &a, int parity,
     G.stream_hi = a.stream_hi;
     G.gather = a.gather != 0;
     G.write_back = a.gather || a.theta > 0;
+    G.err = &a.st->err;
 #if PA_CHECKED
     G.src_limit = a.st->pop;  // the old population (received runs on a shard) until k_finalize
-    G.err = &a.st->err;
 #endif
     return G;
 }
@@ -112,6 +112,7 @@ __device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
                 g = make_int2(s_next, min(a.rpb, s_end - s_next));
                 s_next += a.rpb;
             }
+            if (*(volatile int32_t *)&st->err) g.y = 0;  // a block gave up (PA_ERR_TIMEOUT): no further groups
             s_group = g;
         }
         __syncthreads();
@@ -121,6 +122,7 @@ __device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
         dev::sweep_group_bits<B, MODE, Q, QCAP, LAT>(G, a.L, reinterpret_cast<uint32_t *>(smem4), s_tab, s_queue,
                                                      a.rk0, a.rk1, a.acc);
     }
+    if (threadIdx.x == 0) dev::bulk_stores_done();
     // the last block to end clears the counters for the next launch and writes
     // the step's estimators (a launch of its own took 5.5 us and a gap)
     __threadfence();
