@@ -76,13 +76,14 @@ __global__ void __launch_bounds__(dev::kWeightsThreads) k_batch_weights(const Ba
 __global__ void __launch_bounds__(kChunk) k_batch_counts(const BatchArgs b)
 {
     __shared__ int s_i[32];
+    __shared__ double s_inv[dev::kPoissonTable];
     const int m = run_of_chunk(b.runs, b.M, blockIdx.x);
     const int i = *b.step_counter;
     const StepDev &sp = b.steps[(size_t)i * b.M + m];
     if (!sp.active) return;
     const RunDev &r = b.runs[m];
     dev::counts_body(blockIdx.x - r.chunk0, r.E, r.nbins - 1, r.R0, r.mode, i, r.stream_hi, b.k0, b.k1, sp.wtab,
-                     r.counts, r.local_off, r.blocksum, r.st, s_i);
+                     r.counts, r.local_off, r.blocksum, r.st, s_i, s_inv, b.poisson);
 }
 
 __global__ void __launch_bounds__(kChunk) k_batch_scatter(const BatchArgs b)
@@ -134,6 +135,7 @@ struct pa_batch {
     std::vector<pa::DevState> st_start;
     int32_t *hist_all = nullptr;
     unsigned long long *acc_all = nullptr;
+    double *poisson = nullptr;  // table of full Poisson pieces
     size_t bins_total = 0;
     std::vector<void *> allocs;
     pa::BatchArgs args{};
@@ -477,6 +479,7 @@ pa_status pa_batch_create(const pa_run_desc *runs, int32_t M, void *cuda_stream,
         take(&b->st_all, M);
         take(&b->hist_all, b->bins_total);
         take(&b->acc_all, 3 * (size_t)M);
+        take(&b->poisson, pa::kPoissonTableEntries);
     };
     lay_out();
     if ((s = balloc(b, &arena, arena_bytes))) return fail(s);
@@ -570,6 +573,10 @@ pa_status pa_batch_create(const pa_run_desc *runs, int32_t M, void *cuda_stream,
         a.rk1[r] = a.k1 + 0xBB67AE85u * (uint32_t)r;
     }
     a.gather = 1;
+    a.poisson = nullptr;
+    for (const pa_config &g : b->cfg)
+        if (g.resample_mode == PA_RESAMPLE_POISSON) a.poisson = b->poisson;
+    if (a.poisson && (e = pa::launch_poisson_table(b->poisson, b->stream)) != cudaSuccess) return fail(bfail(e));
     int budget = 65536;
     for (int m = 0; m < M; ++m) budget = std::max(budget, (int)pa::replica_bytes(b->cfg[m].q, b->cfg[m].L));
     if ((s = balloc(b, &b->stage, stage_bytes))) return fail(s);

@@ -46,6 +46,7 @@ struct BatchArgs {
     long long total_items;
     uint32_t k0, k1;
     uint32_t rk0[10], rk1[10];
+    const double *poisson;  // table of full Poisson pieces (null: no run draws any)
     int32_t gather;  // 0 for the measurement at step 0
 };
 

@@ -113,6 +113,7 @@ struct pa_ctx {
     uint8_t *stage = nullptr;
     size_t stage_bytes = 0;
     uint8_t *host_stage = nullptr;  // pinned: device state, one record, the histogram
+    double *poisson = nullptr;  // table of full Poisson pieces (PA_RESAMPLE_POISSON only)
     double *aux = nullptr;  // small device outputs (Newton step)
     int hist_span = 0;      // bins from the lowest to the highest occupied one at the last pa_next_dbeta
     int32_t *hstore = nullptr;  // histograms taken by pa_run
@@ -295,7 +296,7 @@ void release(pa_ctx *c)
     if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
     void *ptrs[] = {c->spins[0], c->spins[1], c->anc[0], c->anc[1], c->E, c->Mt, c->hist, c->fam,
                     c->counts, c->local_off, c->blocksum, c->parent, c->acc, c->st, c->obs,
-                    c->stage, c->aux, c->hstore, c->work};
+                    c->stage, c->aux, c->poisson, c->hstore, c->work};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (c->host_stage) cudaFreeHost(c->host_stage);
@@ -535,7 +536,7 @@ pa_status enqueue_resample(pa_ctx *c, double dbeta, int step, int table = 0)
     if ((s = profile_mark(c, 1, true))) return s;
     PA_CK(pa::launch_resample(c->hist, c->nbins, c->E, dbeta, c->cfg.R, c->R_cap, c->cfg.resample_mode, step,
                               (uint32_t)c->cfg.stream << 24, c->k0, c->k1, wtab, c->counts, c->local_off,
-                              c->blocksum, c->parent, c->hist, c->st, c->stream));
+                              c->blocksum, c->parent, c->hist, c->st, c->stream, 0, 0, nullptr, nullptr, c->poisson));
     if ((s = profile_mark(c, 1, false))) return s;
     c->pending_step = step;
     c->resampled = true;
@@ -657,6 +658,10 @@ pa_status ctx_create(const pa_config &g, void *cuda_stream, pa_ctx **out, int ra
         return fail(s);
     e = cudaMemsetAsync(c->work, 0, 2 * sizeof(int32_t), c->stream);
     if (e != cudaSuccess) return fail(cuda_fail(e));
+    if (g.resample_mode == PA_RESAMPLE_POISSON) {
+        if ((s = dev_alloc(&c->poisson, pa::kPoissonTableEntries))) return fail(s);
+        if ((e = pa::launch_poisson_table(c->poisson, c->stream)) != cudaSuccess) return fail(cuda_fail(e));
+    }
     if (g.track_families) {
         if ((s = dev_alloc(&c->anc[0], c->R_cap)) || (s = dev_alloc(&c->anc[1], c->R_cap)) ||
             (s = dev_alloc(&c->fam, g.R)))
@@ -1190,7 +1195,8 @@ pa_status pa_shard_counts(pa_ctx *c, double dbeta, int32_t step, int64_t *local_
     if (s) return s;
     PA_CK(pa::launch_resample(c->hist, c->nbins, c->E, dbeta, c->cfg.R, c->cfg.R_cap, c->cfg.resample_mode, step,
                               (uint32_t)c->cfg.stream << 24, c->k0, c->k1, wtab, c->counts, c->local_off,
-                              c->blocksum, c->parent, c->hist, c->st, c->stream, c->slot0, c->R_all));
+                              c->blocksum, c->parent, c->hist, c->st, c->stream, c->slot0, c->R_all, nullptr, nullptr,
+                              c->poisson));
     pa::DevState h;
     s = sync_state(c, &h);
     if (s == PA_ERR_CAPACITY) {

@@ -146,7 +146,12 @@ cudaError_t launch_resample(const int32_t *hist, int nbins, const int32_t *E, do
                             int R_cap, int mode, int step, uint32_t stream_hi, uint32_t k0, uint32_t k1,
                             const double *wtab, int32_t *counts, int32_t *local_off, int32_t *blocksum,
                             int32_t *parent, int32_t *hist_zero, DevState *st, cudaStream_t s, int j0 = 0,
-                            int R_prev_all = 0, double *lnQ_out = nullptr, int32_t *R_out = nullptr);
+                            int R_prev_all = 0, double *lnQ_out = nullptr, int32_t *R_out = nullptr,
+                            const double *poisson_full = nullptr);
+// The table of full Poisson pieces (kPoissonTableEntries doubles) that
+// launch_resample may be given.
+constexpr int kPoissonTableEntries = 256;
+cudaError_t launch_poisson_table(double *F, cudaStream_t s);
 // R_all: size of the whole population when the sums cover several GPUs (0 otherwise).
 cudaError_t launch_finalize(DevState *st, unsigned long long *acc, int32_t *fam, int R0, DevObs *obs,
                             double beta, int q, int N, int gathered, int resampled, cudaStream_t s, int R_all = 0);

@@ -519,12 +519,45 @@ __device__ __forceinline__ void weights_body(const int32_t *hist, int nbins, dou
     cl.sync();  // the blocks' limbs stay until the first has read them
 }
 
+// Cumulative probabilities F_n of a full piece (mean 64) of a Poisson draw, by
+// the recursion of poisson_draw; one thread, once.
+constexpr double kPoissonPiece = 64.0;
+constexpr int kPoissonTable = kPoissonTableEntries;
+__device__ __forceinline__ void poisson_table(double *F_out)
+{
+    double p = exp(-kPoissonPiece), F = p;
+    F_out[0] = F;
+    for (int n = 1; n < kPoissonTable; ++n) {
+        p = __ddiv_rn(__dmul_rn(p, kPoissonPiece), (double)n);
+        F = __dadd_rn(F, p);
+        F_out[n] = F;
+    }
+}
+
+// inv[n] = 1 / n for n = 1 .. kPoissonTable - 1, by the whole block.
+__device__ __forceinline__ void reciprocals(double *inv)
+{
+    for (int n = threadIdx.x; n < kPoissonTable; n += blockDim.x) inv[n] = n ? __ddiv_rn(1.0, (double)n) : 0.0;
+}
+
 // A Poisson draw with mean rho for replica j (Sec. 2, Eq. 1): inversion of
 // the cumulative distribution with the mean split into pieces of at most 64;
 // the k-th uniform (U_k + 1/2) / 2^32 is word k & 3 of counter
 // (j, RESAMPLE | (1 + k / 4), step, stream).
+//
+// Bound by the serial chain of the replicas with the largest means (a population
+// with a few families has copy numbers of hundreds: 149 us per launch for 5003
+// replicas).  Full pieces share one cumulative table (full, null: none), in
+// which the result is found by bisection -- the recursion visits F_0 .. F_n in
+// rising order, so of the near-tie tests only those of F_{n-1} and F_n can
+// differ from the rest.  The others divide by n < 256 through inv[n] = 1 / n and
+// one residual (Markstein, IBM J. Res. Dev. 34, 1990): q = x inv is within two
+// units in the last place of x / n, x - q n is exact in a fused operation, and
+// q + (x - q n) inv misses x / n by less than 2^-50 units before it is rounded,
+// while x / n stays 1 / (2 n) units away from every midpoint: the result is the
+// quotient correctly rounded, and every F_n the double that the division gives.
 __device__ __forceinline__ int poisson_draw(double rho, int j, int step, uint32_t stream_hi, uint32_t k0, uint32_t k1,
-                                            bool &tie)
+                                            const double *inv, const double *full, bool &tie)
 {
     int r = 0;
     tie = false;
@@ -532,12 +565,23 @@ __device__ __forceinline__ int poisson_draw(double rho, int j, int step, uint32_
     uint32_t k = 0;
     uint4 w = make_uint4(0u, 0u, 0u, 0u);
     while (remaining > 0.0) {
-        const double mu = remaining < 64.0 ? remaining : 64.0;
+        const double mu = remaining < kPoissonPiece ? remaining : kPoissonPiece;
         remaining = __dsub_rn(remaining, mu);
         if ((k & 3) == 0)
             w = philox10(make_uint4((uint32_t)j, DOM_RESAMPLE | (1u + (k >> 2)), (uint32_t)step, stream_hi), k0, k1);
-        const double u = __ddiv_rn(__dadd_rn((double)pick_word(w, k & 3), 0.5), 4294967296.0);
+        const double u = __dmul_rn(__dadd_rn((double)pick_word(w, k & 3), 0.5), 0x1p-32);
         k += 1;
+        if (full && mu == kPoissonPiece && u <= full[kPoissonTable - 1]) {
+            int lo = 0, hi = kPoissonTable - 1;  // the first n with u <= F_n
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (u > full[mid]) lo = mid + 1; else hi = mid;
+            }
+            if (fabs(__dsub_rn(u, full[lo])) < 0x1p-40) tie = true;
+            if (lo > 0 && fabs(__dsub_rn(u, full[lo - 1])) < 0x1p-40) tie = true;
+            r += lo;
+            continue;
+        }
         double p = exp(-mu);
         double F = p;
         int n = 0;
@@ -545,7 +589,13 @@ __device__ __forceinline__ int poisson_draw(double rho, int j, int step, uint32_
             if (fabs(__dsub_rn(u, F)) < 0x1p-40) tie = true;
             if (!(u > F && n < 1000)) break;
             n += 1;
-            p = __ddiv_rn(__dmul_rn(p, mu), (double)n);
+            const double x = __dmul_rn(p, mu);
+            if (n < kPoissonTable) {
+                const double q = __dmul_rn(x, inv[n]);
+                p = __fma_rn(__fma_rn(-q, (double)n, x), inv[n], q);
+            } else {
+                p = __ddiv_rn(x, (double)n);
+            }
             F = __dadd_rn(F, p);
         }
         r += n;
@@ -570,11 +620,15 @@ __device__ __forceinline__ bool round_tie(double rho, double frac, double bounda
 __device__ __forceinline__ void counts_body(int chunk, const int32_t *E, int twoN, int R_target, int mode, int step,
                                             uint32_t stream_hi, uint32_t k0, uint32_t k1, const double *wtab,
                                             int32_t *counts, int32_t *local_off, int32_t *blocksum, DevState *st,
-                                            int *s_i, int j0 = 0)
+                                            int *s_i, double *s_inv, const double *poisson_full, int j0 = 0)
 {
     if (st->err) return;
     const int R_prev = st->pop;
     if (chunk * (int)blockDim.x >= R_prev) return;
+    if (mode == 2) {
+        reciprocals(s_inv);
+        __syncthreads();
+    }
     const int j = chunk * blockDim.x + threadIdx.x;
     int r = 0;
     bool tie = false;
@@ -586,7 +640,7 @@ __device__ __forceinline__ void counts_body(int chunk, const int32_t *E, int two
         const double frac = __dsub_rn(rho, n);
         const int jg = j0 + j;
         if (mode == 2) {
-            r = poisson_draw(rho, jg, step, stream_hi, k0, k1, tie);
+            r = poisson_draw(rho, jg, step, stream_hi, k0, k1, s_inv, poisson_full, tie);
         } else if (mode == 3) {
             r = 1;
         } else if (mode == 1) {

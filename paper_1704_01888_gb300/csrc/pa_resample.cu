@@ -54,13 +54,19 @@ __global__ void __launch_bounds__(dev::kWeightsThreads) k_weights(const int32_t 
 __global__ void __launch_bounds__(kBlock) k_counts(const int32_t *E, int twoN, int R_target, int mode, int step,
                                                    uint32_t stream_hi, uint32_t k0, uint32_t k1, const double *wtab,
                                                    int32_t *counts, int32_t *local_off, int32_t *blocksum,
-                                                   DevState *st, int j0)
+                                                   DevState *st, int j0, const double *poisson_full)
 {
     __shared__ int s_i[32];
+    __shared__ double s_inv[dev::kPoissonTable];
     launch_dependents();
     wait_prerequisites();
     dev::counts_body(blockIdx.x, E, twoN, R_target, mode, step, stream_hi, k0, k1, wtab, counts, local_off, blocksum,
-                     st, s_i, j0);
+                     st, s_i, s_inv, poisson_full, j0);
+}
+
+__global__ void k_poisson_table(double *F)
+{
+    if (threadIdx.x == 0) dev::poisson_table(F);
 }
 
 __global__ void __launch_bounds__(kBlock) k_scatter(const int32_t *counts, const int32_t *local_off,
@@ -241,7 +247,7 @@ cudaError_t launch_resample(const int32_t *hist, int nbins, const int32_t *E, do
                             int R_cap, int mode, int step, uint32_t stream_hi, uint32_t k0, uint32_t k1,
                             const double *wtab, int32_t *counts, int32_t *local_off, int32_t *blocksum,
                             int32_t *parent, int32_t *hist_zero, DevState *st, cudaStream_t s, int j0,
-                            int R_prev_all, double *lnQ_out, int32_t *R_out)
+                            int R_prev_all, double *lnQ_out, int32_t *R_out, const double *poisson_full)
 {
     const int threads = resample_chunk(R_cap);
     const int nb = (R_cap + threads - 1) / threads;
@@ -249,13 +255,20 @@ cudaError_t launch_resample(const int32_t *hist, int nbins, const int32_t *E, do
                                  dbeta, wtab, st, R_prev_all);
     if (e == cudaSuccess)
         e = launch_after(k_counts, 1, nb, threads, 0, s, E, nbins - 1, R_target, mode, step, stream_hi, k0, k1, wtab,
-                         counts, local_off, blocksum, st, j0);
+                         counts, local_off, blocksum, st, j0, poisson_full);
     // every block clears its share of the histogram too
     if (e == cudaSuccess)
         e = launch_after(k_scatter, 1, nb, threads, 0, s, counts, local_off, blocksum, parent, R_cap, hist_zero, nbins,
                          st, R_prev_all > 0 ? 0 : 1, lnQ_out, R_out);
     bump_launch_count(3);
     return e;
+}
+
+cudaError_t launch_poisson_table(double *F, cudaStream_t s)
+{
+    k_poisson_table<<<1, 32, 0, s>>>(F);
+    bump_launch_count(1);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_finalize(DevState *st, unsigned long long *acc, int32_t *fam, int R0, DevObs *obs,

@@ -406,9 +406,11 @@ __global__ void __launch_bounds__(kNewtonThreads) k_newton_hist(const int32_t *_
 template <typename K>
 int cluster_blocks(K kernel, int threads, size_t smem)
 {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return 0;
-    int best = 8;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return 0;
+    int n = 0;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) {
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -419,11 +421,10 @@ int cluster_blocks(K kernel, int threads, size_t smem)
         cfg.dynamicSmemBytes = smem;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0) best = kClusterMax;
+        e = cudaOccupancyMaxActiveClusters(&n, kernel, &cfg);
     }
-    (void)cudaGetLastError();  // a refused size is no error of the caller's
-    return best;
+    if (e != cudaSuccess) (void)cudaGetLastError();  // a refused size is no error of the caller's
+    return e == cudaSuccess && n > 0 ? kClusterMax : 8;
 }
 
 // The cluster size of a kernel, looked up once per device.

@@ -20,6 +20,20 @@ def _built():
     oracle.build()
 
 
+@pytest.mark.parametrize("R,dbeta", [(700, 0.4), (5003, 0.05), (5003, 0.4), (5003, 2.0), (20000, 1.2)])
+def test_poisson_tables_give_the_oracles_copy_numbers(R, dbeta):
+    """pa_resample draws full Poisson pieces (mean 64) from a table: copy
+    numbers from one to thousands."""
+    cap = 2 * R + 2000
+    with pa.Population(pa.PAParams(q=5, L=16, R=R, seed=4, resample_mode=pa.RESAMPLE_POISSON, R_cap=cap)) as pop:
+        E = pop.energies()
+        lnq, R_new = pop.resample(dbeta, 1, sync=True)
+        r, ref_lnq, ref_R, rho = oracle.copy_numbers(E, dbeta, R, pa.RESAMPLE_POISSON, 1, 4)
+        assert R_new == ref_R and lnq == pytest.approx(ref_lnq, rel=1e-12, abs=1e-12)
+        assert np.array_equal(pop.parents(R_new), oracle.parents(r))
+    assert dbeta < 2.0 or rho.max() > 200.0
+
+
 @pytest.mark.parametrize("R,cap", [(1, 8), (127, 1500), (128, 1500), (129, 1500), (2047, 5000), (2049, 5000),
                                    (5003, 131072), (5003, 131073), (150000, 200000)])
 @pytest.mark.parametrize("L,lo,hi,dbeta", [(64, -4300, -4200, 0.01), (64, -8192, 0, -0.01), (256, -131072, 0, 1e-4),
