@@ -64,6 +64,48 @@ __global__ void __launch_bounds__(kBlock) k_counts(const int32_t *E, int twoN, i
                      st, s_i, s_inv, poisson_full, j0);
 }
 
+// Small populations (capacities up to kSmallResample): the three stages in one
+// cluster, its barriers between them, with the bodies of k_weights, k_counts
+// and k_scatter.  Two launches fewer per step where launches count; larger
+// populations' FP64 work wants more SMs than a cluster has.
+constexpr int kSmallResample = 4096, kSmallThreads = 256;
+__global__ void __launch_bounds__(kSmallThreads) k_resample_small(const int32_t *hist, int nbins, const int32_t *E,
+                                                                  double dbeta, int R_target, int R_cap, int mode,
+                                                                  int step, uint32_t stream_hi, uint32_t k0,
+                                                                  uint32_t k1, const double *wtab, int32_t *counts,
+                                                                  int32_t *local_off, int32_t *blocksum,
+                                                                  int32_t *parent, int32_t *hist_zero, DevState *st,
+                                                                  int j0, int R_prev_all, double *lnQ_out,
+                                                                  int32_t *R_out, const double *poisson_full)
+{
+    __shared__ dev::WeightsShared sh;
+    __shared__ long long s_l[32];
+    __shared__ int s_i[32];
+    __shared__ double s_inv[dev::kPoissonTable];
+    launch_dependents();
+    wait_prerequisites();
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), c = (int)cl.block_rank();
+    dev::weights_body(hist, nbins, dbeta, wtab, st, sh, R_prev_all);  // ends with a cluster barrier
+    const int nb = (R_cap + kSmallThreads - 1) / kSmallThreads;
+    for (int chunk = c; chunk < nb; chunk += C) {
+        dev::counts_body(chunk, E, nbins - 1, R_target, mode, step, stream_hi, k0, k1, wtab, counts, local_off,
+                         blocksum, st, s_i, s_inv, poisson_full, j0);
+        __syncthreads();
+    }
+    cl.sync();
+    const int chunks = max(nb, C);
+    for (int chunk = c; chunk < chunks; chunk += C) {
+        dev::scatter_body(chunk, chunks, counts, local_off, blocksum, parent, R_cap, hist_zero, nbins, st, s_l,
+                          R_prev_all > 0 ? 0 : 1);
+        __syncthreads();
+    }
+    if (R_out && c == 0 && threadIdx.x == 0) {
+        *R_out = st->err ? -st->err : st->pop_next;
+        *lnQ_out = st->err ? 0.0 : st->lnQ;
+    }
+}
+
 __global__ void k_poisson_table(double *F)
 {
     if (threadIdx.x == 0) dev::poisson_table(F);
@@ -249,6 +291,12 @@ cudaError_t launch_resample(const int32_t *hist, int nbins, const int32_t *E, do
                             int32_t *parent, int32_t *hist_zero, DevState *st, cudaStream_t s, int j0,
                             int R_prev_all, double *lnQ_out, int32_t *R_out, const double *poisson_full)
 {
+    if (R_cap <= kSmallResample) {
+        bump_launch_count(1);
+        return launch_after(k_resample_small, kWeightsCluster, kWeightsCluster, kSmallThreads, 0, s, hist, nbins, E,
+                            dbeta, R_target, R_cap, mode, step, stream_hi, k0, k1, wtab, counts, local_off, blocksum,
+                            parent, hist_zero, st, j0, R_prev_all, lnQ_out, R_out, poisson_full);
+    }
     const int threads = resample_chunk(R_cap);
     const int nb = (R_cap + threads - 1) / threads;
     cudaError_t e = launch_after(k_weights, kWeightsCluster, kWeightsCluster, dev::kWeightsThreads, 0, s, hist, nbins,
