@@ -378,8 +378,9 @@ const char *pa_last_cuda_error(void);
 /* Launch-shape control for the sweep kernel: replicas per block and threads
  * per block (0 = automatic).  Any choice gives bit-identical results; this
  * exists for autotuning and for tests that check exactly that.  Automatic:
- * 96 KB of lattices and up to 512 threads per block (two blocks per SM), or,
- * for L = 128 and 256 with states of at most five bits and at least 16
+ * the blocks per SM, rounds and threads with the least modelled time, the
+ * population in even shares, or,
+ * for L = 128 (up to eight rounds) and 256 with states of at most five bits and at least 16
  * replicas per SM, one block of 1024 threads per SM holding as many whole
  * passes of lattices as fit 200 KB.  Errors: PA_ERR_INVALID for a shape that
  * does not fit (threads not a multiple of 32 or above 1024, lattices above
