@@ -9,12 +9,15 @@
 //               S of the Boltzmann factors w = exp(-dbeta (E - E_ref)) (taken
 //               from a table the host computes with the C library's exp;
 //               summed exactly and rounded once) and
-//               ln Q_i = -dbeta E_ref + ln(S/R_{i-1}).
+//               ln Q_i = -dbeta E_ref + ln(S/R_{i-1}); one cluster.
 //   k_counts    copy numbers r_j from rho_j = R w(E_j) / S and their
 //               block-local exclusive scan (warp shuffles).
 //   k_scatter   block offsets, the new population size R_i (checked against
 //               the capacity) and the parent map parent[off_j + c] = j.
-//   k_finalize  Sec. 2 step 4 / Sec. 3 Eq. 4: population averages from exact
+//   k_resample_small  the three stages above in one cluster, for capacities
+//               of at most 4096 replicas.
+//   k_finalize  (with families and for shares of a population; otherwise the
+//               sweep's last block does this) Sec. 2 step 4 / Sec. 3 Eq. 4: population averages from exact
 //               integer sums, the fluctuation-formula specific heat, the
 //               magnetisation of Eq. 5, ln Z of Eq. 2 and the family entropy.
 // All floating-point steps that feed a decision (S, rho, the rounding test)

@@ -128,7 +128,7 @@ __device__ __forceinline__ void cluster_sum(cg::cluster_group &cl, double (&v)[N
 // cluster and evaluates one exp per occupied bin.  The observable's sums read
 // {w, w e} per replica from a table that the blocks fill in one another's
 // shared memory, two fused multiply-adds each.  Otherwise (few replicas, or
-// energies spread wider than the table) one exp per replica, as before.
+// energies spread wider than the table) one exp per replica.
 // One launch of one cluster: no workspace to allocate, share or clear.  Now
 // 12.8 us for R = 2e5 (two readings of E and three cluster barriers) and 17.0 us
 // for 1e5 with an observable (12 more bytes per replica through 16 SMs).
