@@ -333,7 +333,10 @@ double half_sweep_cost(bool lat, int k, int rpb, long long units, int threads)
     const BlockWork w = block_work(rpb, units, threads);
     const double resident = k * threads / 32.0, measured = 0.03 * rpb / (threads / 32.0);
     if (lat) return 1.0 + measured + std::max(0.078 * (double)(k * w.warps), 0.4 * (double)w.passes);
-    const double slack = 1.0 + 0.2 * std::max(0.0, 32.0 - resident) / 32.0;
+    // a block's warps spread over four schedulers: ten load two of them with three
+    const int bw = threads / 32;
+    const double uneven = bw > 4 ? 0.5 * ((bw + 3) / 4 * 4 - bw) / bw : 0.0;
+    const double slack = 1.0 + 0.2 * std::max(0.0, 32.0 - resident) / 32.0 + uneven;
     return 0.9 + 1.0 / k + measured + std::max(0.074 * slack * (double)(k * w.warps), 0.6 * (double)w.passes);
 }
 
