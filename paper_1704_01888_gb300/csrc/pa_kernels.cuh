@@ -667,11 +667,17 @@ __device__ __forceinline__ void counts_body(int chunk, const int32_t *E, int two
 // min_total: smallest valid number of children (1; 0 for one GPU's share of
 // a population spread over several, which may receive all its replicas from
 // the others).
+//
+// Every block takes the capacity decision from its own sum over the chunks.
+// Chunk 0's block records a refusal in st->err while others may still be
+// reading the flag here, so a block's threads vote on what they read: each on
+// its own, some would leave and the rest meet the wrong barriers and use the
+// stale sums of the chunk before as offsets into parent.
 __device__ __forceinline__ void scatter_body(int chunk, int nchunks, const int32_t *counts, const int32_t *local_off,
                                              const int32_t *blocksum, int32_t *parent, int R_cap, int32_t *hist_zero,
                                              int nbins, DevState *st, long long *s_l, int min_total = 1)
 {
-    if (st->err) return;
+    if (__syncthreads_or(*(volatile int32_t *)&st->err)) return;
     const int R_prev = st->pop;
     const int nb = (R_prev + blockDim.x - 1) / blockDim.x;
     long long off = 0, tot = 0;
