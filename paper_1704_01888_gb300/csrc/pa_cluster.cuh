@@ -66,7 +66,7 @@ cudaError_t launch_clusters(void (*kernel)(P...), int C, int blocks, int threads
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+    return launch_result(cudaLaunchKernelEx(&cfg, kernel, (P)args...));
 }
 
 }  // namespace pa

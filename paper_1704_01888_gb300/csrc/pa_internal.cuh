@@ -208,6 +208,14 @@ namespace pa {
 __device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// A launch's error is reported once, by its return value: left pending on the
+// thread as well, it would be taken for a later call's.
+inline cudaError_t launch_result(cudaError_t e)
+{
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+}
+
 template <typename... P, typename... A>
 cudaError_t launch_after(void (*kernel)(P...), int cluster, int blocks, int threads, size_t smem, cudaStream_t s,
                          A... args)
@@ -225,7 +233,7 @@ cudaError_t launch_after(void (*kernel)(P...), int cluster, int blocks, int thre
     cfg.stream = s;
     cfg.attrs = at;
     cfg.numAttrs = cluster > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, (P)args...);
+    return launch_result(cudaLaunchKernelEx(&cfg, kernel, (P)args...));
 }
 
 // Philox4x32-10 (Salmon, Moraes, Dror & Shaw, SC'11): ten rounds of two

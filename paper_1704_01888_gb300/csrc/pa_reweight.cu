@@ -406,8 +406,9 @@ __global__ void __launch_bounds__(kNewtonThreads) k_newton_hist(const int32_t *_
 template <typename K>
 int cluster_blocks(K kernel, int threads, size_t smem)
 {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return 0;
+    cudaError_t e =
+        launch_result(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (e != cudaSuccess) return 0;  // not kept: the next call asks again
     int n = 0;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) {
