@@ -51,7 +51,8 @@ typedef enum {
     PA_ERR_CUDA = 3,     /* a CUDA runtime call failed; see pa_last_cuda_error */
     PA_ERR_TIMEOUT = 4,  /* a block of the sweep kernel waited about a second for
                             its own copies and gave up (its kernels do not wait
-                            on one another)                                   */
+                            on one another).  The context has failed; of a
+                            batch, every run that the launch was to sweep     */
     PA_ERR_STATE = 5,    /* calls in the wrong order, or a failed context      */
     PA_ERR_NOMEM = 6,    /* device or host allocation failed                   */
     PA_ERR_TOO_LARGE = 7 /* a replica larger than one block's shared memory

@@ -618,6 +618,9 @@ pa_status pa_batch_run(pa_batch *b, int32_t use_graph)
     if (!b) return PA_ERR_INVALID;
     if (b->ran) return PA_ERR_STATE;
     b->ran = true;
+#if PA_CHECKED
+    b->args.give_up = pa::give_up_slot();
+#endif
     if (!use_graph) {
         for (int i = 1; i <= b->Kmax; ++i) {
             pa_status s = enqueue_step(b, b->stream);

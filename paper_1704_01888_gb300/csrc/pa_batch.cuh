@@ -48,6 +48,9 @@ struct BatchArgs {
     uint32_t rk0[10], rk1[10];
     const double *poisson;  // table of full Poisson pieces (null: no run draws any)
     int32_t gather;  // 0 for the measurement at step 0
+#if PA_CHECKED
+    int32_t give_up;  // as in SweepArgs
+#endif
 };
 
 // The part of the batched sweep that takes a run's replica groups.
@@ -103,7 +106,7 @@ __global__ void __launch_bounds__(1024) k_batch_sweep(const BatchArgs b)
     extern __shared__ uint4 smem4[];
     __shared__ uint4 s_tab[dev::kThresholdEntries];
     __shared__ int s_prefix[kMaxRuns + 1];
-    __shared__ int s_group;
+    __shared__ int s_group, s_gave_up;
     __shared__ __align__(16) uint32_t s_queue[dev::queue_words(PART == 0 ? 4 : 7)];
     const int i = *b.step_counter;
     int *work = b.work + PART * b.work_stride + i;
@@ -120,11 +123,25 @@ __global__ void __launch_bounds__(1024) k_batch_sweep(const BatchArgs b)
             }
         }
         s_prefix[b.M] = acc;
+        s_gave_up = 0;
     }
     __syncthreads();
     const int total = s_prefix[b.M];
     for (;;) {
-        if (threadIdx.x == 0) s_group = atomicAdd(work, 1);
+        if (threadIdx.x == 0) {
+            if (s_gave_up) {
+                // this block gives up.  Should all, groups would stay undone: no
+                // further one is handed out, and every run of the launch is marked
+                // (in this order: a block that starts late and leaves marked runs
+                // out of its list of groups then finds none left)
+                atomicMax(work, total);
+                __threadfence();
+                for (int k = 0; k < b.M; ++k)
+                    if (batch_part(b.runs[k].q) == PART && b.steps[(size_t)i * b.M + k].active)
+                        atomicCAS(&b.runs[k].st->err, 0, 4);  // PA_ERR_TIMEOUT
+            }
+            s_group = s_gave_up ? total : atomicAdd(work, 1);
+        }
         __syncthreads();
         const int g = s_group;
         __syncthreads();
@@ -161,8 +178,10 @@ __global__ void __launch_bounds__(1024) k_batch_sweep(const BatchArgs b)
         G.gather = b.gather != 0;
         G.write_back = b.gather || sp.theta > 0;
         G.err = &r.st->err;
+        G.gave_up = &s_gave_up;
 #if PA_CHECKED
         G.src_limit = r.st->pop;
+        G.give_up = b.give_up == first + 1;
 #endif
         dev::build_threshold_table(s_tab, sp.thr);
         uint32_t *sw = reinterpret_cast<uint32_t *>(smem4);

@@ -48,6 +48,14 @@ Thresholds acceptance_thresholds(double beta)
     return th;
 }
 
+#if PA_CHECKED
+int give_up_slot()
+{
+    const char *v = std::getenv("PA_CHECKED_GIVE_UP");
+    return v ? std::atoi(v) : 0;
+}
+#endif
+
 void weight_table(double dbeta, int n, double *out)
 {
     for (int t = 0; t < n; ++t) {
@@ -500,6 +508,9 @@ pa::SweepArgs sweep_args(pa_ctx *c, double beta, int theta, int step, int gather
     a.dynamic = R_est < 16LL * c->group * c->grid;
     a.counters = c->work;
     a.beta = beta;
+#if PA_CHECKED
+    a.give_up = pa::give_up_slot();
+#endif
     return a;
 }
 

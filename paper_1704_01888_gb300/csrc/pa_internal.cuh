@@ -120,6 +120,9 @@ struct SweepArgs {
     int32_t *counters;         // next replica group, blocks ended; zero before and after each launch
     DevObs *obs;               // the step's record, written by the last block (null: by launch_finalize)
     double beta;
+#if PA_CHECKED
+    int32_t give_up;           // give_up_slot()
+#endif
 };
 
 // Launchers (pa_sweep.cu)
@@ -192,6 +195,14 @@ cudaError_t launch_newton(const int32_t *hist, int nbins, const DevState *st, do
                           double *out, cudaStream_t s);
 
 int64_t bump_launch_count(int64_t n);
+
+#if PA_CHECKED
+// The replica groups whose wait for bulk copies counts as run out: those that
+// start at slot give_up_slot() - 1 (0: none), from the environment variable
+// PA_CHECKED_GIVE_UP.  The tests' way to the path of PA_ERR_TIMEOUT; the copies
+// themselves arrive.
+int give_up_slot();
+#endif
 
 // Records the message returned by pa_last_cuda_error() on this thread.
 void record_cuda_error(const char *msg);

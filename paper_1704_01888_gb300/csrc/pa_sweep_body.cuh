@@ -272,8 +272,10 @@ struct Group {
     uint32_t stream_hi;      // stream number << 24, or'ed into the slot counter word
     bool gather, write_back;
     int32_t *err;            // the run's error flag
+    int *gave_up;            // shared, set where the block may take no further group (null: it reads err)
 #if PA_CHECKED
     int src_limit;           // a gather's parent slots lie in [0, src_limit)
+    bool give_up;            // a test: count the wait for the bulk copies as run out
 #endif
 };
 
@@ -300,7 +302,8 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
 }
 
 // Waits for the barrier's bytes, at most about a second (kBulkClocks); false if
-// they did not come.
+// they did not come.  Whoever gives up takes no further group: the barrier and
+// the shared memory may still be written by the copies that are late.
 constexpr long long kBulkClocks = 2000000000ll;
 __device__ __forceinline__ bool bulk_wait(uint32_t bar)
 {
@@ -582,6 +585,9 @@ __device__ __forceinline__ void propose(const uint32_t (&W)[BP], const uint32_t 
 // 9387 at q = 20, L = 256, R = 2e4; 4331 -> 4060 at q = 8, L = 128, R = 5e4; 728 ->
 // 635 at q = 6, L = 32, R = 1e5; 761 -> 656 at q = 8, L = 48, R = 5e4; 3769 -> 3390
 // at q = 3, L = 100, R = 5e4.
+//
+// Where the copies into shared memory do not come, G.err becomes PA_ERR_TIMEOUT
+// and the block must leave its loop over the groups.
 template <int B, int MODE, int Q = 0, int QCAP = kQueueCap, bool LAT = false>
 __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32_t *sw, const uint4 *s_tab,
                                                  uint32_t *qbuf, const uint32_t *rk0, const uint32_t *rk1,
@@ -631,12 +637,18 @@ __device__ __forceinline__ void sweep_group_bits(const Group &G, int Lrt, uint32
         } else {
             for (int r = tid; r < nrep; r += blockDim.x) bulk_load(shared_address(sw + r * RW), source(r), RB, bar);
         }
-        const bool ok = bulk_wait(bar);
-        if (__syncthreads_or(!ok)) {
+        bool here = bulk_wait(bar);
+#if PA_CHECKED
+        here = here && !G.give_up;
+#endif
+        if (__syncthreads_or(!here)) {
             // not expected to happen: report it, give the copies once more the
             // time to land, and leave the group
-            if (tid == 0) atomicExch(G.err, 4);  // PA_ERR_TIMEOUT
-            bulk_wait(bar);
+            if (tid == 0) {
+                atomicExch(G.err, 4);  // PA_ERR_TIMEOUT
+                if (G.gave_up) *G.gave_up = 1;
+                bulk_wait(bar);
+            }
             __syncthreads();
             return;
         }

@@ -46,8 +46,10 @@ __device__ __forceinline__ dev::Group make_group(const SweepArgs &a, int parity,
     G.gather = a.gather != 0;
     G.write_back = a.gather || a.theta > 0;
     G.err = &a.st->err;
+    G.gave_up = nullptr;
 #if PA_CHECKED
     G.src_limit = a.st->pop;  // the old population (received runs on a shard) until k_finalize
+    G.give_up = a.give_up == first + 1;
 #endif
     return G;
 }
@@ -88,7 +90,6 @@ __device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
     dev::build_threshold_table(s_tab, a.thr);
     wait_prerequisites();
     DevState *st = a.st;
-    if (st->err) return;
     const int parity = st->parity;
     // thread 0 hands out the groups from shared memory: nothing of it stays in
     // registers through the sweeps
@@ -112,7 +113,10 @@ __device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
                 g = make_int2(s_next, min(a.rpb, s_end - s_next));
                 s_next += a.rpb;
             }
-            if (*(volatile int32_t *)&st->err) g.y = 0;  // a block gave up (PA_ERR_TIMEOUT): no further groups
+            // the run has failed, before this launch or by a block that gave up
+            // (PA_ERR_TIMEOUT; this one too): no group, and every block still counts
+            // itself below
+            if (*(volatile int32_t *)&st->err) g.y = 0;
             s_group = g;
         }
         __syncthreads();
@@ -130,7 +134,7 @@ __device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
     if (threadIdx.x == 0 && atomicAdd(a.counters + 1, 1) == (int)gridDim.x - 1) {
         __threadfence();
         a.counters[0] = a.counters[1] = 0;
-        if (a.obs && !st->err)
+        if (a.obs && !*(volatile int32_t *)&st->err)
             dev::finalize_record(st, a.acc, a.obs, a.beta, a.q, a.L * a.L, a.gather, a.gather, 0, 0.0, 0);
     }
 }
