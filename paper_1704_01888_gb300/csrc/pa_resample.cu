@@ -246,20 +246,29 @@ __global__ void k_shard_check(DevState *st, int expected)
     if (threadIdx.x == 0 && blockIdx.x == 0 && !st->err && st->pop_next != expected) st->err = 1;  // PA_ERR_INVALID
 }
 
-__global__ void k_to_canonical(const uint32_t *spins, uint8_t *out, int q, int L, long long count)
+// Bytes from the planes: 64 sites per thread where words_in_order (k_canonical_words),
+// else one site per thread (k_canonical_sites).
+__global__ void k_canonical_words(const uint32_t *spins, uint8_t *out, int q, int L, long long count)
 {
-    if (dev::words_in_order(L) && (reinterpret_cast<uintptr_t>(out) & 15) == 0) {
-        const long long total = count * colour_words(L);
-        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-             i += (long long)gridDim.x * blockDim.x)
-            dev::canonical_words(spins, out, q, L, i);
-        return;
-    }
+    const long long total = count * colour_words(L);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+         i += (long long)gridDim.x * blockDim.x)
+        dev::canonical_words(spins, out, q, L, i);
+}
+
+__global__ void k_canonical_sites(const uint32_t *spins, uint8_t *out, int q, int L, long long count)
+{
     const long long total = count * L * L;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x)
         out[i] = dev::canonical_state(spins, q, L, i);
 }
+
+// Smallest readout that takes k_canonical_words.  One thread's 64 sites are a
+// chain of about 2 us that a short readout does not hide: at q = 10 and 40 one site
+// per thread takes 5.8 us against 7.8 up to 2^17 sites, 7.8 against 7.8 at 2^18,
+// and 14 against 7.8 at 2^20 (launch included).
+constexpr int64_t kCanonicalWordSites = 1 << 18;
 
 __global__ void k_from_canonical(uint32_t *spins, const uint8_t *canon, int q, int L, long long count)
 {
@@ -332,7 +341,11 @@ cudaError_t launch_finalize(DevState *st, unsigned long long *acc, int32_t *fam,
 
 cudaError_t launch_to_canonical(const uint32_t *spins, uint8_t *out, int q, int L, int64_t count, cudaStream_t s)
 {
-    k_to_canonical<<<grid_for(dev::words_in_order(L) ? count * colour_words(L) : count * L * L, 256), 256, 0, s>>>(spins, out, q, L, count);
+    const int64_t sites = count * L * L;
+    if (dev::words_in_order(L) && sites >= kCanonicalWordSites && (reinterpret_cast<uintptr_t>(out) & 15) == 0)
+        k_canonical_words<<<grid_for(count * colour_words(L), 256), 256, 0, s>>>(spins, out, q, L, count);
+    else
+        k_canonical_sites<<<grid_for(sites, 256), 256, 0, s>>>(spins, out, q, L, count);
     bump_launch_count(1);
     return cudaGetLastError();
 }
