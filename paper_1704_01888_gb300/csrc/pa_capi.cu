@@ -448,6 +448,13 @@ pa_status choose_launch(pa_ctx *c, int rpb_req, int threads_req)
         int rpb_fill = c->R_fill / (4 * c->sms);
         if (rpb_fill < 1) rpb_fill = 1;
         rpb = rpb_mem < rpb_fill ? rpb_mem : rpb_fill;
+        // whole passes of 512 threads over the site words (q = 10, L = 64 with 256
+        // threads, R = 6000: 8 replicas 159 us, 9 164), at least a warp of words
+        // (q = 6, L = 32 with 512 threads, R = 1000: two replicas 72 us, one 103)
+        const long long per_pass = 512 / units;
+        if (per_pass >= 1 && rpb > per_pass) rpb = (int)(rpb / per_pass * per_pass);
+        const int rpb_warp = (int)((32 + units - 1) / units);
+        if (rpb < rpb_warp) rpb = std::min(rpb_warp, rpb_mem);
     }
     if ((size_t)rpb * RB > (size_t)pa::kMaxLatticeBytes) return rpb == 1 ? PA_ERR_TOO_LARGE : PA_ERR_INVALID;
     if (threads <= 0) {
@@ -457,8 +464,10 @@ pa_status choose_launch(pa_ctx *c, int rpb_req, int threads_req)
     }
     if (threads % 32 != 0 || threads > 1024) return PA_ERR_INVALID;
     const long long groups = ((long long)c->R_cap + rpb - 1) / rpb;
-    // the latency kernel where its blocks are all resident at once
-    bool lat = threads <= 512 && groups * threads <= 512LL * c->sms;
+    // the latency kernel where its blocks are all resident at once and a thread
+    // has one site word (six words: 193 us against 184 at q = 10, L = 64, blocks
+    // of 48 replicas and 512 threads)
+    bool lat = threads <= 512 && groups * threads <= 512LL * c->sms && block_work(rpb, units, threads).passes <= 1;
     int per_sm = pa::sweep_max_blocks_per_sm(c->cfg.q, L, rpb, threads, lat);
     if (per_sm <= 0 && lat) {
         lat = false;

@@ -1,0 +1,60 @@
+"""Launch shapes of which the caller gives one number, and groups handed out
+from the counter over more than three rounds, whose last half round goes out in
+half groups."""
+import numpy as np
+import pytest
+
+import paper_1704_01888_gb300 as pa
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_1704_01888_gb300 import build
+
+    build.build()
+
+
+def _shape(q, L, R, launch):
+    with pa.Population(pa.PAParams(q=q, L=L, R=R, seed=1)) as pop:
+        pop.set_launch(*launch)
+        return pop.launch_shape()
+
+
+def test_threads_alone_fill_their_warps_and_passes():
+    """At least a warp of site words to a block; whole passes of 512 threads."""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for threads in (256, 512):
+        assert _shape(6, 32, 1000, (0, threads))[:2] == (2, threads)  # 16 words per colour
+        assert _shape(2, 8, 1000, (0, threads))[:2] == (32, threads)  # one word per colour
+        # ten replicas of 64 words would be a pass and a quarter
+        assert _shape(10, 64, 40 * sms, (0, threads))[:2] == (8, threads)
+    assert _shape(20, 256, 100, (0, 512))[0] == 1
+
+
+@pytest.mark.parametrize("q,L,rpb,threads", [(10, 32, 6, 32), (3, 16, 20, 32), (2, 8, 40, 32), (20, 48, 5, 64),
+                                             (5, 100, 4, 416), (6, 64, 8, 128)])
+def test_half_groups_give_the_same_population(q, L, rpb, threads):
+    """Sizes that divide into neither the groups nor the halves."""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    betas = np.array([0.0, 0.5, 1.0])
+
+    def run(R, launch):
+        with pa.Population(pa.PAParams(q=q, L=L, R=R, seed=2)) as pop:
+            pop.set_launch(*launch)
+            shape = pop.launch_shape()
+            obs, _ = pop.run(betas, 1)
+            return shape, [(o["R"], o["sumE"], o["sumE2"], o["sumMt"]) for o in obs], pop.energies(), pop.spins()
+
+    blocks = _shape(q, L, 1000000 // (L * L // 64), (rpb, threads))[2]  # as many as fit the GPU
+    assert blocks % sms == 0
+    R = 3 * blocks * rpb + blocks * rpb // 3 + 1
+    shape, obs, E, spins = run(R, (rpb, threads))
+    assert shape == (rpb, threads, blocks) and 3 * blocks * rpb < min(o[0] for o in obs) and R < 16 * blocks * rpb
+    other = run(R, (max(1, rpb // 2), 2 * threads))
+    assert obs == other[1] and np.array_equal(E, other[2]) and np.array_equal(spins, other[3])
