@@ -236,17 +236,22 @@ class Clocks:
                 "samples": len(sm)}
 
 
+# every file of this package that pa_sweep.cu is compiled from
+SWEEP_SOURCES = ("pa_sweep.cu", "pa_sweep_kernel.cuh", "pa_kernels.cuh", "pa_cluster.cuh", "pa_sweep_body.cuh",
+                 "pa_internal.cuh")
+
+
 def _sweep_sources() -> bytes:
     csrc = os.path.join(ROOT, "paper_1704_01888_gb300", "csrc")
-    return b"".join(open(os.path.join(csrc, f), "rb").read()
-                    for f in ("pa_sweep.cu", "pa_sweep_kernel.cuh", "pa_sweep_body.cuh", "pa_internal.cuh"))
+    return b"".join(open(os.path.join(csrc, f), "rb").read() for f in SWEEP_SOURCES)
 
 
-def _sweep_record(w):
+def _sweep_record(w, launch):
     """The sweep kernel's ncu record (profiles/sweep_traffic.txt): DRAM bytes
     per replica per launch and the issue activity, valid only for the
-    workload's (q, L) it was taken on and while the sweep kernel's sources
-    hash to the recorded value."""
+    workload's (q, L) and the launch shape (replicas and threads per block,
+    blocks) it was taken on and while the sweep kernel's sources hash to the
+    recorded value."""
     rec = {}
     try:
         for line in open(os.path.join(ROOT, "profiles", "sweep_traffic.txt")):
@@ -258,7 +263,7 @@ def _sweep_record(w):
         return None
     if rec.get("source_sha256") != hashlib.sha256(_sweep_sources()).hexdigest():
         return None
-    if rec.get("case") != f"q{w.q}-L{w.L}":
+    if rec.get("case") != f"q{w.q}-L{w.L}" or rec.get("launch") != ",".join(str(x) for x in launch):
         return None
     out = {"dram_bytes_per_replica": float(rec["dram_bytes_per_replica"])}
     if "issue_active" in rec:
@@ -425,7 +430,7 @@ def run_ours(args):
     opa = ops_per_attempt(w.q, A, w.theta)
     achieved = opa * per_launch_attempts / sweep_avg_s / 1e12
     peak = sms * LANES_PER_SM_PER_CLK * f_max / 1e12
-    rec = _sweep_record(w)
+    rec = _sweep_record(w, launch_used)
     per_launch_replicas = per_launch_attempts / (w.N * w.theta)
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s", "frac": achieved / peak,
                 "traffic": (rec["dram_bytes_per_replica"] * per_launch_replicas) if rec else None,
