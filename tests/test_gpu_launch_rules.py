@@ -58,3 +58,24 @@ def test_half_groups_give_the_same_population(q, L, rpb, threads):
     assert shape == (rpb, threads, blocks) and 3 * blocks * rpb < min(o[0] for o in obs) and R < 16 * blocks * rpb
     other = run(R, (max(1, rpb // 2), 2 * threads))
     assert obs == other[1] and np.array_equal(E, other[2]) and np.array_equal(spins, other[3])
+
+
+@pytest.mark.parametrize("L,R", [(8, 1), (8, 100000), (16, 1000), (32, 10000), (48, 50000), (64, 1), (64, 151),
+                                 (64, 153), (64, 1000), (64, 20000), (64, 100000), (96, 3000), (100, 5003),
+                                 (100, 30000), (128, 1000), (192, 3000), (256, 600)])
+def test_automatic_shape_is_an_even_share(L, R):
+    """A block's replicas are the share of a round of all the blocks that an SM
+    holds, for the population with the spread of its copy numbers."""
+    import math
+
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    with pa.Population(pa.PAParams(q=8, L=L, R=R, seed=1)) as pop:
+        rpb, threads, blocks = pop.launch_shape()
+    planned = R + 2 * math.ceil(math.sqrt(R))
+    slots = -(-blocks // sms) * sms
+    rounds = -(-planned // (slots * rpb))
+    assert rpb == -(-planned // (slots * rounds))
+    assert blocks == min(slots, -(-planned // rpb))
+    assert threads % 32 == 0 and 32 <= threads <= 1024
