@@ -336,6 +336,10 @@ BlockWork block_work(int rpb, long long units, int threads)
 // Fitted to launches of theta = 10 at q = 10, L = 64: 3.6, 5.5 and 11.6 us per
 // half sweep for 28, 56 and 136 warp passes per SM.  The latency kernel
 // (lat) takes 2.2 us for 14 and 1.3 us for 2 where the other takes 2.3 and 1.6.
+// The constants serve every plane count and row geometry: over 460 random sizes
+// the shapes take 0.69 times the time of blocks of 512 threads and 96 KB
+// (geometric mean), more in seven of them, 6 % at most (q = 2 and 3, L = 32, R =
+// 9700; one to three planes cost less per warp pass than the four fitted).
 double half_sweep_cost(bool lat, int k, int rpb, long long units, int threads)
 {
     const BlockWork w = block_work(rpb, units, threads);
@@ -449,8 +453,9 @@ pa_status choose_launch(pa_ctx *c, int rpb_req, int threads_req)
         if (rpb_fill < 1) rpb_fill = 1;
         rpb = rpb_mem < rpb_fill ? rpb_mem : rpb_fill;
         // whole passes of 512 threads over the site words (q = 10, L = 64 with 256
-        // threads, R = 6000: 8 replicas 159 us, 9 164), at least a warp of words
-        // (q = 6, L = 32 with 512 threads, R = 1000: two replicas 72 us, one 103)
+        // threads, R = 6000: 144 us a launch of theta = 10 with 8 replicas, 164 with
+        // 9), at least a warp of words (q = 6, L = 32 with 512 threads, R = 1000: 60
+        // us with two replicas, 103 with one)
         const long long per_pass = 512 / units;
         if (per_pass >= 1 && rpb > per_pass) rpb = (int)(rpb / per_pass * per_pass);
         const int rpb_warp = (int)((32 + units - 1) / units);
@@ -465,7 +470,7 @@ pa_status choose_launch(pa_ctx *c, int rpb_req, int threads_req)
     if (threads % 32 != 0 || threads > 1024) return PA_ERR_INVALID;
     const long long groups = ((long long)c->R_cap + rpb - 1) / rpb;
     // the latency kernel where its blocks are all resident at once and a thread
-    // has one site word (six words: 193 us against 184 at q = 10, L = 64, blocks
+    // has one site word (six words: 193 us against 163 at q = 10, L = 64, blocks
     // of 48 replicas and 512 threads)
     bool lat = threads <= 512 && groups * threads <= 512LL * c->sms && block_work(rpb, units, threads).passes <= 1;
     int per_sm = pa::sweep_max_blocks_per_sm(c->cfg.q, L, rpb, threads, lat);

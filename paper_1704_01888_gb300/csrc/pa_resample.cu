@@ -17,8 +17,9 @@
 //   k_resample_small  the three stages above in one cluster, for capacities
 //               of at most 4096 replicas.
 //   k_finalize  (with families and for shares of a population; otherwise the
-//               sweep's last block does this) Sec. 2 step 4 / Sec. 3 Eq. 4: population averages from exact
-//               integer sums, the fluctuation-formula specific heat, the
+//               sweep's last block does this) Sec. 2 step 4 / Sec. 3 Eq. 4:
+//               population averages from exact integer sums, the
+//               fluctuation-formula specific heat, the
 //               magnetisation of Eq. 5, ln Z of Eq. 2 and the family entropy.
 // All floating-point steps that feed a decision (S, rho, the rounding test)
 // use explicitly rounded operations so that no multiply-add is contracted.

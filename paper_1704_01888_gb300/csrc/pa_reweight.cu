@@ -469,10 +469,9 @@ pa_status pa_reweight_forward(const int32_t *E, const double *O, int32_t R, cons
     // a small population does not fill a cluster: one block per 1024 replicas
     int blocks = C;
     while (blocks > 1 && (long long)(blocks / 2) * 1024 >= R) blocks /= 2;
-    return pa::launch_clusters(pa::k_rw_forward, blocks, blocks, pa::kRwThreads, smem, (cudaStream_t)stream, E, O, R, dbeta,
-                              out) == cudaSuccess
-               ? PA_OK
-               : PA_ERR_CUDA;
+    const cudaError_t e = pa::launch_clusters(pa::k_rw_forward, blocks, blocks, pa::kRwThreads, smem,
+                                              (cudaStream_t)stream, E, O, R, dbeta, out);
+    return e == cudaSuccess ? PA_OK : PA_ERR_CUDA;
 }
 
 pa_status pa_reweight_scale(const double *src, int32_t idx, double sign, const double *g, double *dst, void *stream)

@@ -390,7 +390,8 @@ constexpr int kThresholdFull = 40;
 // planes takes 384 entries (its 48 lattices give up to ~250 queued words at
 // low temperature, so 256 entries overflowed: 1846 against 1837 attempts/ns
 // over the at-scale schedule; two blocks per SM still fit); the batched kernel
-// keeps 256, whose 96 KB lattice budget two blocks per SM would not fit with more.
+// keeps 256: more gave 3104 against 3124 PA steps/s in blocks of 96 KB of
+// lattices, and its default blocks hold a third of those.
 constexpr int kFirstPassCalls = 2;
 constexpr int kLatCalls = 3;
 constexpr int kLatQueue = 90;
@@ -565,9 +566,10 @@ __device__ __forceinline__ void propose(const uint32_t (&W)[BP], const uint32_t 
 
 // Multi-spin-coded sweep body.  B = bits per state (compile time), MODE as
 // for neighbour_planes, Q = q when fixed at compile time (0: q from G).  Each
-// loop step of a thread updates one site word: 32 same-colour sites.  The random numbers follow this rule: in
-// sweep k, colour c, the site word with index w = y WPR + t draws the stream
-// Z_0, Z_1, ... (Z_{4n+i} = word i of the Philox call with counter
+// loop step of a thread updates one site word: 32 same-colour sites.  The
+// random numbers follow this rule: in sweep k, colour c, the site word with
+// index w = y WPR + t draws the stream Z_0, Z_1, ... (Z_{4n+i} = word i of the
+// Philox call with counter
 // (w, SWEEP | (2k + c) << 8 | n, step, slot | stream)); the site at bit b takes
 // bit b of each: direction sigma from Z_0, offset u from Z_1..Z_{B-1}, and
 // acceptance bits v_j from Z_{B+j}, most significant first.  Proposal
@@ -576,14 +578,15 @@ __device__ __forceinline__ void propose(const uint32_t (&W)[BP], const uint32_t 
 // indicator bits (neighbours equal to s, neighbours different from s'), summed
 // by a carry-save tree; moves with dE > 0 compare v with T[dE] bit by bit.
 //
-// Bound by issue: the logic runs on the ALU pipe (half a warp instruction per
-// clock and scheduler), the Philox products on the FMA-heavy one (a quarter).
-// What is made once per word, per word index or per half sweep is therefore
-// kept out of the 378 instructions per word (409 before the shared Philox
-// rounds, the shorter proposal and the smaller queue entries).  Launches of
-// theta = 10 next to beta_t: 2104 -> 2064 us at q = 10, L = 64, R = 1e5; 9722 ->
-// 9387 at q = 20, L = 256, R = 2e4; 4331 -> 4060 at q = 8, L = 128, R = 5e4; 728 ->
-// 635 at q = 6, L = 32, R = 1e5; 761 -> 656 at q = 8, L = 48, R = 5e4; 3769 -> 3390
+// Bound by the ALU pipe (half a warp instruction per clock and scheduler; 65 %
+// busy at q = 10, L = 64, R = 65536) and beside it the FMA-heavy one (a quarter),
+// which takes the Philox products.  What is made once per word, per word index
+// or per half sweep is therefore kept out of the 362 instructions per word (409
+// before the shared Philox rounds, the shorter proposal and the smaller queue
+// entries).  Launches of theta = 10 next to beta_t, with 409 instructions and the
+// launch shapes of then against now: 2138 -> 1979 us at q = 10, L = 64, R = 1e5;
+// 9721 -> 8097 at q = 20, L = 256, R = 2e4; 4359 -> 3820 at q = 8, L = 128, R = 5e4; 743
+// -> 525 at q = 6, L = 32, R = 1e5; 774 -> 595 at q = 8, L = 48, R = 5e4; 3782 -> 3041
 // at q = 3, L = 100, R = 5e4.
 //
 // Where the copies into shared memory do not come, G.err becomes PA_ERR_TIMEOUT

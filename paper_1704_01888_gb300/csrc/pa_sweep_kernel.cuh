@@ -58,8 +58,8 @@ __device__ __forceinline__ dev::Group make_group(const SweepArgs &a, int parity,
 // of rpb replicas, and in launches of more than three rounds the last half
 // round's worth in halves (whole passes each).  With whole groups to the end a
 // block that took its last one late held the launch up by half a round: 2043 or
-// 2178 us from step to step at q = 10, L = 64, R = 1e5 (6.86 rounds), now
-// 2050.  Returns the first replica (R or more: no group left) and the size.
+// 2178 us from step to step at q = 10, L = 64, R = 1e5 (6.86 rounds), 2015 with
+// halves.  Returns the first replica (R or more: no group left) and the size.
 __device__ __forceinline__ int2 ticket_range(int t, int R, int rpb, int quantum, int blocks)
 {
     const long long round = (long long)blocks * rpb;
