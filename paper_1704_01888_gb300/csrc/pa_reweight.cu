@@ -234,8 +234,10 @@ __global__ void __launch_bounds__(kRwThreads) k_rw_forward(const int32_t *__rest
             const double mO = __ddiv_rn(v[4], S);
             const double mO_lo = __ddiv_rn(__fma_rn(-mO, S, v[4]), S);
             const double p = __dmul_rn(mO, v[1]), p_lo = __fma_rn(mO, v[1], -p);
+            const double cov = __ddiv_rn(__dsub_rn(__dsub_rn(__dsub_rn(v[5], p), p_lo), __dmul_rn(mO_lo, v[1])), S);
             out[3] = mO;
-            out[4] = __ddiv_rn(__dsub_rn(__dsub_rn(__dsub_rn(v[5], p), p_lo), __dmul_rn(mO_lo, v[1])), S);
+            // sums that overflow have no residuals
+            out[4] = isfinite(cov) ? cov : __dsub_rn(__ddiv_rn(v[5], S), __dmul_rn(mO, m1));
         }
         out[5] = (double)ref;
         out[6] = S;

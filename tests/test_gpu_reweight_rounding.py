@@ -84,3 +84,29 @@ def test_sums_over_the_cluster_round_no_more_than_in_one_block():
         one.append([(s[0] - S) / S, (s[2] / s[0] - mO) / mO, (s[3] / s[0] - (s[2] / s[0]) * (s[1] / s[0]) - cov) / scale])
     lib, one = (np.sqrt((np.array(x, dtype=LD) ** 2).mean(axis=0)) for x in (lib, one))
     assert np.all(lib <= 1.16 * one), (lib, one)
+
+
+@pytest.mark.parametrize("R,big", [(300, 1e304), (30000, 1e302)])
+def test_covariance_of_observables_beyond_the_doubles(R, big):
+    """sum w O e above the largest double: infinite, as SOe / S - <O> <e> is; an
+    infinite or undefined O leaves no number."""
+    import torch
+    from paper_1704_01888_gb300 import autograd as ag
+
+    E = np.random.default_rng(R).integers(-9000, -4000, size=R).astype(np.int32)
+    E[0] = -9000
+    d = torch.tensor(1e-5, dtype=torch.float64, device="cuda")
+
+    def cov(O):
+        out = ag.reweight_forward(torch.tensor(E, device="cuda"), d, torch.tensor(O, device="cuda")).cpu().numpy()
+        return out[3], out[4]
+
+    mean, c = cov(np.full(R, big))
+    assert mean == pytest.approx(big, rel=1e-14) and c == np.inf
+    mean, c = cov(np.full(R, -big))
+    assert mean == pytest.approx(-big, rel=1e-14) and c == -np.inf
+    for bad in (np.inf, np.nan):
+        O = np.ones(R)
+        O[R // 2] = bad
+        mean, c = cov(O)
+        assert (mean == bad or np.isnan(bad) and np.isnan(mean)) and np.isnan(c)
