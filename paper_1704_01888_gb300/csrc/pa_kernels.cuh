@@ -670,17 +670,18 @@ __device__ __forceinline__ void counts_body(int chunk, const int32_t *E, int two
 //
 // Every block takes the capacity decision from its own sum over the chunks.
 // Chunk 0's block records a refusal in st->err while others may still be
-// reading the flag here, so a block's threads vote on what they read: each on
-// its own, some would leave and the rest meet the wrong barriers and use the
-// stale sums of the chunk before as offsets into parent.
+// reading the flag here: threads that each went by their own reading could
+// leave some of the block's barriers to the rest, which would use the stale
+// sums of the chunk before as offsets into parent.  So thread 0 alone reads it,
+// and what it saw reaches the others as part of the sum.
 __device__ __forceinline__ void scatter_body(int chunk, int nchunks, const int32_t *counts, const int32_t *local_off,
                                              const int32_t *blocksum, int32_t *parent, int R_cap, int32_t *hist_zero,
                                              int nbins, DevState *st, long long *s_l, int min_total = 1)
 {
-    if (__syncthreads_or(*(volatile int32_t *)&st->err)) return;
+    const bool failed = threadIdx.x == 0 && *(volatile int32_t *)&st->err;
     const int R_prev = st->pop;
     const int nb = (R_prev + blockDim.x - 1) / blockDim.x;
-    long long off = 0, tot = 0;
+    long long off = 0, tot = failed ? 1ll << 60 : 0;
     for (int b = threadIdx.x; b < nb; b += blockDim.x) {
         const long long v = blocksum[b];
         tot += v;
@@ -689,7 +690,7 @@ __device__ __forceinline__ void scatter_body(int chunk, int nchunks, const int32
     tot = block_sum_ll(tot, s_l);
     off = block_sum_ll(off, s_l);
     if (tot > R_cap || tot < min_total) {
-        if (chunk == 0 && threadIdx.x == 0) st->err = 2;  // PA_ERR_CAPACITY
+        if (chunk == 0 && threadIdx.x == 0 && !failed) st->err = 2;  // PA_ERR_CAPACITY
         return;
     }
     if (chunk == 0 && threadIdx.x == 0) st->pop_next = (int)tot;
