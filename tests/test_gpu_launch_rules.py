@@ -79,3 +79,21 @@ def test_automatic_shape_is_an_even_share(L, R):
     assert rpb == -(-planned // (slots * rounds))
     assert blocks == min(slots, -(-planned // rpb))
     assert threads % 32 == 0 and 32 <= threads <= 1024
+
+
+@pytest.mark.parametrize("lattices,shape", [((16, 64), (32768, 256)), ((40,), (32768, 256)), ((96, 100), (131072, 1024)),
+                                            ((18, 66), (131072, 1024)), ((256,), (65536, 512))])
+def test_batch_shape_follows_the_words_that_threads_find(lattices, shape):
+    """Few and many of 256 threads without a site word; the runs are lone runs."""
+    betas = np.array([0.0, 0.5, 1.0])
+    runs = [(pa.PAParams(q=q, L=L, R=300, seed=4, stream=m), betas, 2)
+            for m, (q, L) in enumerate((q, L) for L in lattices for q in (3, 10))]
+    with pa.Batch(runs) as b:
+        assert b.launch_shape()[:2] == shape
+        b.run()
+        for m, (p, _, _) in enumerate(runs):
+            with pa.Population(p) as pop:
+                obs, _ = pop.run(betas, 2)
+                E, Mt = b.measurements(m)
+                assert b.observables(m)[1:] == obs
+                assert np.array_equal(E, pop.energies()) and np.array_equal(Mt, pop.occupations())
