@@ -214,8 +214,13 @@ namespace pa {
 // Programmatic dependent launch: the kernels of a temperature step are launched
 // while their predecessor runs (launch_after), so that a launch costs little
 // between them.  A kernel so launched calls wait_prerequisites() before it
-// touches memory; it may let its own successor start at any time, since that
-// waits for it in turn.
+// touches memory.  Its successor waits in turn and could start at any time; it
+// is let in (launch_dependents) as a block's work ends.  Let in at once, the next
+// sweep's blocks came while the sweep before still ran, and the SMs that
+// happened to be free took several of the few blocks that are to be spread
+// evenly: 108 steps of q = 8, L = 48, R = 832 (149 blocks) took 6.1 or 7.4 ms from
+// build to build, now 5.9; back to back sweeps of q = 3, L = 64, R = 664 44.5 us, now
+// 35.4.
 __device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

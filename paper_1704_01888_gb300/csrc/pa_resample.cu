@@ -50,9 +50,9 @@ __global__ void __launch_bounds__(dev::kWeightsThreads) k_weights(const int32_t 
                                                                   const double *wtab, DevState *st, int R_prev_all)
 {
     __shared__ dev::WeightsShared sh;
-    launch_dependents();
     wait_prerequisites();
     dev::weights_body(hist, nbins, dbeta, wtab, st, sh, R_prev_all);
+    launch_dependents();
 }
 
 __global__ void __launch_bounds__(kBlock) k_counts(const int32_t *E, int twoN, int R_target, int mode, int step,
@@ -62,10 +62,10 @@ __global__ void __launch_bounds__(kBlock) k_counts(const int32_t *E, int twoN, i
 {
     __shared__ int s_i[32];
     __shared__ double s_inv[dev::kPoissonTable];
-    launch_dependents();
     wait_prerequisites();
     dev::counts_body(blockIdx.x, E, twoN, R_target, mode, step, stream_hi, k0, k1, wtab, counts, local_off, blocksum,
                      st, s_i, s_inv, poisson_full, j0);
+    launch_dependents();
 }
 
 // Small populations (capacities up to kSmallResample): the three stages in one
@@ -86,7 +86,6 @@ __global__ void __launch_bounds__(kSmallThreads) k_resample_small(const int32_t 
     __shared__ long long s_l[32];
     __shared__ int s_i[32];
     __shared__ double s_inv[dev::kPoissonTable];
-    launch_dependents();
     wait_prerequisites();
     cg::cluster_group cl = cg::this_cluster();
     const int C = (int)cl.num_blocks(), c = (int)cl.block_rank();
@@ -108,6 +107,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_resample_small(const int32_t 
         *R_out = st->err ? -st->err : st->pop_next;
         *lnQ_out = st->err ? 0.0 : st->lnQ;
     }
+    launch_dependents();
 }
 
 __global__ void k_poisson_table(double *F)
@@ -121,7 +121,6 @@ __global__ void __launch_bounds__(kBlock) k_scatter(const int32_t *counts, const
                                                     double *lnQ_out, int32_t *R_out)
 {
     __shared__ long long s_l[32];
-    launch_dependents();
     wait_prerequisites();
     dev::scatter_body(blockIdx.x, gridDim.x, counts, local_off, blocksum, parent, R_cap, hist_zero, nbins, st, s_l,
                       min_total);
@@ -129,6 +128,7 @@ __global__ void __launch_bounds__(kBlock) k_scatter(const int32_t *counts, const
         *R_out = st->err ? -st->err : st->pop_next;
         *lnQ_out = st->err ? 0.0 : st->lnQ;
     }
+    launch_dependents();
 }
 
 __global__ void __launch_bounds__(kBlock) k_finalize(DevState *st, unsigned long long *acc, int32_t *fam, int R0,

@@ -86,7 +86,6 @@ __device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
     __shared__ uint4 s_tab[dev::kThresholdEntries];
     constexpr int QCAP = LAT ? dev::kLatQueue : B <= 4 ? 384 : dev::kQueueCap;
     __shared__ __align__(16) uint32_t s_queue[dev::queue_words(B, QCAP)];
-    launch_dependents();
     dev::build_threshold_table(s_tab, a.thr);
     wait_prerequisites();
     DevState *st = a.st;
@@ -126,6 +125,7 @@ __device__ __forceinline__ void sweep_blocks(const SweepArgs &a)
         dev::sweep_group_bits<B, MODE, Q, QCAP, LAT>(G, a.L, reinterpret_cast<uint32_t *>(smem4), s_tab, s_queue,
                                                      a.rk0, a.rk1, a.acc);
     }
+    launch_dependents();
     if (threadIdx.x == 0) dev::bulk_stores_done();
     // the last block to end clears the counters for the next launch and writes
     // the step's estimators (a launch of its own took 5.5 us and a gap)
