@@ -336,10 +336,11 @@ BlockWork block_work(int rpb, long long units, int threads)
 // Fitted to launches of theta = 10 at q = 10, L = 64: 3.6, 5.5 and 11.6 us per
 // half sweep for 28, 56 and 136 warp passes per SM.  The latency kernel
 // (lat) takes 2.2 us for 14 and 1.3 us for 2 where the other takes 2.3 and 1.6.
-// The constants serve every plane count and row geometry: over 460 random sizes
-// the shapes take 0.69 times the time of blocks of 512 threads and 96 KB
-// (geometric mean), more in seven of them, 6 % at most (q = 2 and 3, L = 32, R =
-// 9700; one to three planes cost less per warp pass than the four fitted).
+// The constants serve every plane count and row geometry: over 610 random sizes
+// the shapes take 0.70 times the time of blocks of 512 threads and 96 KB
+// (geometric mean), more in ten of them, 8 % at most (600 to 1100 replicas of L =
+// 192 and 256, where the planned spread of R costs a round or a fifth of the SMs;
+// q = 2 and 3, L = 32, R = 9700: fewer planes than the four fitted).
 double half_sweep_cost(bool lat, int k, int rpb, long long units, int threads)
 {
     const BlockWork w = block_work(rpb, units, threads);
